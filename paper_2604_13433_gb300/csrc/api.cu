@@ -617,6 +617,8 @@ packsell_status packsell_spmv_backward(const packsell_matrix *A, const float *x,
         return fail(PACKSELL_ERR_INVALID_ARG,
                     "packsell_spmv_backward: dval needs a matrix encoded with keep_rowptr");
     cudaStream_t s = as_stream(stream);
+    // both results in one pass over the words where a kernel takes them together
+    if (dx && dval && backward_fused(*M(A))) return backward_impl(*M(A), 1.0f, dy, x, dx, dval, s);
     if (dx) {
         const packsell_status st = spmv_t_impl(*M(A), dy, dx, s);
         if (st != PACKSELL_OK) return st;

@@ -163,6 +163,16 @@ packsell_status launch_split_batch(const SplitMat *mats, const MultiItem *items,
 packsell_status launch_split(const Matrix &A, const void *perm, int pb, const float *x, float *y,
                              cudaStream_t s);
 
+packsell_status launch_split_backward(const Matrix &A, float alpha, const float *dy, const float *x,
+                                      float *dx, float *out, cudaStream_t s);
+
+// backward.cu: dx = A^T dy (when dx) and out = alpha dy_i x_j on the pattern
+// (when out; needs A.rowptr) in one pass over the words, for the matrices
+// that backward_fused accepts
+bool backward_fused(const Matrix &A);
+packsell_status backward_impl(const Matrix &A, float alpha, const float *dy, const float *x, float *dx,
+                              float *out, cudaStream_t s);
+
 packsell_status launch_stage(const Matrix &A, int v, const void *perm, int pb, const float *x,
                              float *y, cudaStream_t s);
 

@@ -409,6 +409,217 @@ __global__ void __launch_bounds__(SW * 32, 3)
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+
+// ---- backward products (sigma = 1: storage order is CSR order) ----
+// The items and the column scan of the SpMV above; every word with a value
+// adds value * dy_row to dx at its column, and (DV) alpha * dy_row * x goes
+// to the value's place in CSR order. A tile's values are consecutive there,
+// so they are collected in shared memory by their rank among the tile's
+// values and written 32 consecutive ones at a time. The thread-per-row
+// kernels that this replaces walked a row of up to thousands of words on
+// one lane.
+template <int FMT, bool DX, bool DV>
+__device__ __forceinline__ void back_words(const uint32_t (&wd)[8], const uint32_t (&col)[8],
+                                           const float (&g)[8], float alpha, Decode dc,
+                                           const float *__restrict__ x, float *__restrict__ dx,
+                                           float *__restrict__ out, long long q0, long long qend,
+                                           int lane, float *__restrict__ s_val, int &nval) {
+    int cnt = 0;
+    float xv[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        xv[j] = 0.f;
+        if ((wd[j] & 1u) && PS_IN_RANGE(col[j], dc.xlen)) {
+            if (DV) xv[j] = __ldg(x + col[j]);
+            if (DX && g[j] != 0.f) atomicAdd(dx + col[j], split_value<FMT>(wd[j], dc) * g[j]);
+        }
+        cnt += (int)(wd[j] & 1u);
+    }
+    if (!DV) return;
+    int inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    int t = inc - cnt;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        if (wd[j] & 1u) s_val[t++] = (alpha * g[j]) * xv[j];
+    nval = __shfl_sync(0xffffffffu, inc, 31);
+    __syncwarp();
+    for (int k = lane; k < nval; k += 32)
+        if (PS_IN_RANGE(q0 + k, qend)) __stcs(out + q0 + k, s_val[k]);
+    __syncwarp();
+}
+
+template <int FMT, bool DX, bool DV>
+__global__ void __launch_bounds__(SW * 32, 3)
+    k_back_split(int k_left, const int64_t *__restrict__ offset, const uint32_t *__restrict__ pack,
+                 Decode dc, const SplitItem *__restrict__ items, int nitems,
+                 const int64_t *__restrict__ rowptr, float alpha, const float *__restrict__ dy,
+                 const float *__restrict__ x, float *__restrict__ dx, float *__restrict__ out) {
+    __shared__ __align__(16) uint32_t s_lft[SW][ST];             // kAbs | left at row starts
+    __shared__ __align__(16) float s_g[SW][ST];                  // dy of the row at row starts
+    __shared__ __align__(16) float s_val[DV ? SW : 1][DV ? ST : 1];
+    __shared__ __align__(16) uint32_t s_off[SW][2][SR_MAX + 4];
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    int it = gw;
+    if (it >= nitems) return;
+    SplitItem d = items[it], dn{0, 0, 0};
+    if (it + nwarps < nitems) dn = items[it + nwarps];
+    uint4 wv[2];
+    split_load_item(pack, d, lane, wv);
+    split_prefetch_offsets(d, true, offset, s_off[wl][0], lane);
+    int buf = 0;
+    for (; it < nitems; it += nwarps) {
+        const bool has_next = it + nwarps < nitems;
+        SplitItem dnn{0, 0, 0};
+        if (it + 2 * nwarps < nitems) dnn = items[it + 2 * nwarps];
+        uint4 wn[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+        if (has_next) split_load_item(pack, dn, lane, wn);
+        split_prefetch_offsets(dn, has_next, offset, s_off[wl][buf ^ 1], lane);
+        cp_async_wait_older();
+        __syncwarp();
+        const long long a0 = d.base & ~3ll;
+        const int lead = (int)(d.base - a0);
+        uint32_t wd[8], col[8];
+        float g[8];
+        int nval = 0;
+        if (d.meta < 0) {  // one long row, ST words at a time
+            const int row = d.r0, nwd = -d.meta, lim = lead + nwd;
+            const float gr = dy[row];
+            long long q = DV ? rowptr[row] : 0;
+            const long long qend = DV ? rowptr[row + 1] : 0;
+            uint32_t carry = (uint32_t)max(row - k_left, 0);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) g[j] = gr;
+            for (int k0 = 0; k0 < lim; k0 += ST) {
+                uint4 nx[2];
+                split_load(pack, a0 + k0 + ST, lim - k0 - ST, lane, nx);
+                unpack8(wv, wd);
+                uint32_t acc = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int p = k0 + 8 * lane + j;
+                    if ((unsigned)(p - lead) >= (unsigned)nwd) wd[j] = 0u;
+                    acc += split_delta(wd[j], dc);
+                    col[j] = acc;
+                }
+                uint32_t inc = acc;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += v;
+                }
+                const uint32_t before = carry + inc - acc;
+                carry += __shfl_sync(0xffffffffu, inc, 31);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) col[j] += before;
+                back_words<FMT, DX, DV>(wd, col, g, alpha, dc, x, dx, out, q, qend, lane,
+                                        s_val[DV ? wl : 0], nval);
+                q += nval;
+                wv[0] = nx[0];
+                wv[1] = nx[1];
+            }
+        } else {  // a tile of rows
+            const int nrows = d.meta >> 16, nwd = d.meta & 0xFFFF;
+            const uint32_t *soff = s_off[wl][buf];
+            uint4 *lft4 = reinterpret_cast<uint4 *>(s_lft[wl]);
+            lft4[2 * lane] = make_uint4(0, 0, 0, 0);
+            lft4[2 * lane + 1] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+            const uint32_t a0lo = (uint32_t)a0;
+            for (int k = lane; k < nrows; k += 32) {
+                const uint32_t o0 = soff[k], o1 = soff[k + 1];
+                if (o1 != o0) {
+                    const int pos = (int)(o0 - a0lo), r = d.r0 + k;
+                    s_lft[wl][pos] = kAbs | (uint32_t)max(r - k_left, 0);
+                    s_g[wl][pos] = dy[r];
+                }
+            }
+            __syncwarp();
+            uint32_t hl[8], acc = 0;
+            const uint4 l0 = lft4[2 * lane], l1 = lft4[2 * lane + 1];
+            hl[0] = l0.x; hl[1] = l0.y; hl[2] = l0.z; hl[3] = l0.w;
+            hl[4] = l1.x; hl[5] = l1.y; hl[6] = l1.z; hl[7] = l1.w;
+            unpack8(wv, wd);
+            int last = -1;  // the lane's last row start
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int p = 8 * lane + j;
+                if ((unsigned)(p - lead) >= (unsigned)nwd) wd[j] = 0u;
+                acc = col_comb(acc, hl[j] + split_delta(wd[j], dc));
+                col[j] = acc;
+                if (hl[j]) last = p;
+            }
+            uint32_t inc = acc;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc = col_comb(v, inc);
+            }
+            uint32_t exc = __shfl_up_sync(0xffffffffu, inc, 1);
+            if (lane == 0) exc = 0u;
+            // the row that the lane's first words belong to starts in the
+            // nearest earlier lane that holds a row start
+            const unsigned heads = __ballot_sync(0xffffffffu, last >= 0) & ((1u << lane) - 1u);
+            const int from = heads ? 31 - __clz((int)heads) : lane;
+            const int hp = __shfl_sync(0xffffffffu, last, from);
+            float gr = heads ? s_g[wl][hp] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (hl[j]) gr = s_g[wl][8 * lane + j];
+                g[j] = gr;
+                col[j] = col_comb(exc, col[j]) & ~kAbs;
+            }
+            const long long q0 = DV ? rowptr[d.r0] : 0, qend = DV ? rowptr[d.r0 + nrows] : 0;
+            back_words<FMT, DX, DV>(wd, col, g, alpha, dc, x, dx, out, q0, qend, lane,
+                                    s_val[DV ? wl : 0], nval);
+        }
+        __syncwarp();
+        d = dn;
+        dn = dnn;
+        wv[0] = wn[0];
+        wv[1] = wn[1];
+        buf ^= 1;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+template <int FMT, bool DX, bool DV>
+packsell_status launch_back_split(const Matrix &A, float alpha, const float *dy, const float *x,
+                                  float *dx, float *out, cudaStream_t s) {
+    // persistent grid: every block resident at once (cached per process)
+    static std::atomic<int> cached{0};
+    int blocks = cached.load(std::memory_order_relaxed);
+    if (!blocks) {
+        int dev = 0, sms = 0, per = 0;
+        PS_CUDA(cudaGetDevice(&dev));
+        PS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_back_split<FMT, DX, DV>, SW * 32, 0));
+        blocks = sms * std::max(per, 1);
+        cached.store(blocks, std::memory_order_relaxed);
+    }
+    blocks = std::min(blocks, (A.split_nitems + SW - 1) / SW);
+    const int kl = (int)std::min<int64_t>(A.p.k_left, INT32_MAX);
+    k_back_split<FMT, DX, DV><<<blocks, SW * 32, 0, s>>>(
+        kl, A.offset, A.pack, make_decode(A), reinterpret_cast<const SplitItem *>(A.split_items),
+        A.split_nitems, A.rowptr, alpha, dy, x, dx, out);
+    PS_LAUNCH_CHECK("packsell backward product (split rows)");
+    return PACKSELL_OK;
+}
+
+template <int FMT>
+packsell_status launch_back_split_fmt(const Matrix &A, float alpha, const float *dy, const float *x,
+                                      float *dx, float *out, cudaStream_t s) {
+    if (dx && out) return launch_back_split<FMT, true, true>(A, alpha, dy, x, dx, out, s);
+    if (dx) return launch_back_split<FMT, true, false>(A, alpha, dy, x, dx, out, s);
+    return launch_back_split<FMT, false, true>(A, alpha, dy, x, dx, out, s);
+}
+
 template <bool SORTED>
 int split_batch_blocks() {
     static std::atomic<int> cached{0};
@@ -535,6 +746,13 @@ packsell_status launch_split_batch(const SplitMat *mats, const MultiItem *items,
     else k_spmv_split_batch<false><<<blocks, SW * 32, 0, s>>>(mats, items, nitems);
     PS_LAUNCH_CHECK("packsell_batch_spmv (split rows)");
     return PACKSELL_OK;
+}
+
+packsell_status launch_split_backward(const Matrix &A, float alpha, const float *dy, const float *x,
+                                      float *dx, float *out, cudaStream_t s) {
+    return A.p.format == PACKSELL_FMT_FP16
+               ? launch_back_split_fmt<PACKSELL_FMT_FP16>(A, alpha, dy, x, dx, out, s)
+               : launch_back_split_fmt<PACKSELL_FMT_E8MY>(A, alpha, dy, x, dx, out, s);
 }
 
 packsell_status launch_split(const Matrix &A, const void *perm, int pb, const float *x, float *y,

@@ -1224,6 +1224,7 @@ packsell_status spmv_f64_impl(const Matrix &A, const double *x, double *y, cudaS
 }
 
 packsell_status spmv_t_impl(const Matrix &A, const float *dy, float *dx, cudaStream_t s) {
+    if (backward_fused(A)) return backward_impl(A, 1.f, dy, nullptr, dx, nullptr, s);
     if (A.m > 0) PS_CUDA(cudaMemsetAsync(dx, 0, sizeof(float) * A.m, s));
     if (A.n == 0) return PACKSELL_OK;
     const void *perm = A.p.explicit_perm ? nullptr : A.perm;
@@ -1255,6 +1256,7 @@ packsell_status pattern_outer_impl(const Matrix &A, float alpha, const float *u,
         return fail(PACKSELL_ERR_INVALID_ARG,
                     "packsell_pattern_outer: matrix was encoded without keep_rowptr");
     if (A.n == 0 || A.nnz == 0) return PACKSELL_OK;
+    if (backward_fused(A)) return backward_impl(A, alpha, u, v, nullptr, out, s);
     const void *perm = A.perm;  // rows are addressed in original order here
     int pb = A.perm_bytes;
     int g = grid_for(A.n);
