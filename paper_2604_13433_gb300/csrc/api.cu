@@ -154,7 +154,6 @@ packsell_status packsell_encode(const packsell_params *params, int64_t n, int64_
 packsell_status packsell_destroy(packsell_matrix *A) {
     clear_error();
     if (!A) return PACKSELL_OK;
-    cudaDeviceSynchronize();
     destroy_matrix(reinterpret_cast<Matrix *>(A));
     return PACKSELL_OK;
 }
@@ -298,8 +297,8 @@ packsell_status packsell_import(const void *h_blob, size_t bytes, void *stream,
         destroy_matrix(A);
         return st;
     };
-    if (cudaMalloc(&A->offset, 8 * (h.n_slices + 1)) != cudaSuccess ||
-        (h.perm_bytes && cudaMalloc(&A->perm, (size_t)h.perm_bytes * h.n) != cudaSuccess))
+    if (pool_get(&A->offset, 8 * (h.n_slices + 1), s) != cudaSuccess ||
+        (h.perm_bytes && pool_get(&A->perm, (size_t)h.perm_bytes * h.n, s) != cudaSuccess))
         return bail(fail(PACKSELL_ERR_NO_MEMORY, "packsell_import: allocation"));
     if (cudaMemcpyAsync(A->offset, src, 8 * (h.n_slices + 1), cudaMemcpyHostToDevice, s) != cudaSuccess)
         return bail(fail(PACKSELL_ERR_CUDA, "packsell_import: copy"));
@@ -312,26 +311,26 @@ packsell_status packsell_import(const void *h_blob, size_t bytes, void *stream,
     }
     size_t nw = (size_t)std::max<int64_t>(h.n_words, 1);
     if (is_w64(p.format)) {
-        if (cudaMalloc(&A->pack64, 8 * nw) != cudaSuccess)
+        if (pool_get(&A->pack64, 8 * nw, s) != cudaSuccess)
             return bail(fail(PACKSELL_ERR_NO_MEMORY, "packsell_import: allocation"));
         if (cudaMemcpyAsync(A->pack64, src, 8 * (size_t)h.n_words, cudaMemcpyHostToDevice, s) !=
             cudaSuccess)
             return bail(fail(PACKSELL_ERR_CUDA, "packsell_import: copy"));
     } else if (is_w16(p.format)) {
-        if (cudaMalloc(&A->pack16, 2 * nw) != cudaSuccess)
+        if (pool_get(&A->pack16, 2 * nw, s) != cudaSuccess)
             return bail(fail(PACKSELL_ERR_NO_MEMORY, "packsell_import: allocation"));
         if (cudaMemcpyAsync(A->pack16, src, 2 * (size_t)h.n_words, cudaMemcpyHostToDevice, s) !=
             cudaSuccess)
             return bail(fail(PACKSELL_ERR_CUDA, "packsell_import: copy"));
     } else if (is_packed(p.format) || is_fixed(p.format)) {
-        if (cudaMalloc(&A->pack, 4 * (nw + kWordTail)) != cudaSuccess)
+        if (pool_get(&A->pack, 4 * (nw + kWordTail), s) != cudaSuccess)
             return bail(fail(PACKSELL_ERR_NO_MEMORY, "packsell_import: allocation"));
         if (cudaMemcpyAsync(A->pack, src, 4 * (size_t)h.n_words, cudaMemcpyHostToDevice, s) !=
             cudaSuccess)
             return bail(fail(PACKSELL_ERR_CUDA, "packsell_import: copy"));
     } else {
         const size_t eb = vb - 4;
-        if (cudaMalloc(&A->val, eb * nw) != cudaSuccess || cudaMalloc(&A->col, 4 * nw) != cudaSuccess)
+        if (pool_get(&A->val, eb * nw, s) != cudaSuccess || pool_get(&A->col, 4 * nw, s) != cudaSuccess)
             return bail(fail(PACKSELL_ERR_NO_MEMORY, "packsell_import: allocation"));
         if (cudaMemcpyAsync(A->val, src, eb * (size_t)h.n_words, cudaMemcpyHostToDevice, s) !=
                 cudaSuccess ||

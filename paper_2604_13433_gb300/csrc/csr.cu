@@ -206,8 +206,8 @@ int csr_blocks() {
 
 }  // namespace
 
-void csr_plan_free(Matrix &A) {
-    cudaFree(A.csr_items);
+void csr_plan_free(Matrix &A, const Release &rel) {
+    rel(A.csr_items);
     A.csr_items = nullptr;
     A.csr_nitems = 0;
 }
@@ -217,7 +217,6 @@ void csr_plan_free(Matrix &A) {
 // rows; a row of more than CL words is an item of its own. Built on the host
 // from the row offsets.
 packsell_status plan_csr(Matrix &A, cudaStream_t s) {
-    csr_plan_free(A);
     if (!is_packed(A.p.format) || A.p.C != 1 || A.n == 0) return PACKSELL_OK;
     std::vector<int64_t> off((size_t)A.n + 1);
     PS_CUDA(cudaMemcpyAsync(off.data(), A.offset, sizeof(int64_t) * (A.n + 1),
@@ -249,7 +248,7 @@ packsell_status plan_csr(Matrix &A, cudaStream_t s) {
         return off[a.y] - off[a.x] > off[b.y] - off[b.x];
     });
     if (items.size() >= (size_t)INT32_MAX) return fail(PACKSELL_ERR_RANGE, "plan_csr: too many items");
-    PS_CUDA(cudaMalloc(&A.csr_items, sizeof(int2) * items.size()));
+    PS_CUDA(pool_get(&A.csr_items, sizeof(int2) * items.size(), s));
     PS_CUDA(cudaMemcpyAsync(A.csr_items, items.data(), sizeof(int2) * items.size(),
                             cudaMemcpyHostToDevice, s));
     PS_CUDA(cudaStreamSynchronize(s));

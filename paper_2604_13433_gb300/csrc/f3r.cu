@@ -463,7 +463,7 @@ packsell_status run_f3r(const Matrix &A1, const Matrix &A2, const Matrix &A3, co
         256 * 40;
     double *r = nullptr, *ax = nullptr, *zt = nullptr, *prhs = nullptr, *pout = nullptr;
     double nb = 0.0;
-    if (cudaMallocAsync(&mem, need, s) != cudaSuccess) {
+    if (pool_get(&mem, need, s) != cudaSuccess) {
         st = fail(PACKSELL_ERR_NO_MEMORY, "packsell_f3r: workspace allocation");
         goto out;
     }
@@ -616,7 +616,7 @@ done:
 out:
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
-    if (mem) cudaFreeAsync(mem, s);
+    if (mem) pool_put(mem, s);
     cudaStreamSynchronize(s);
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);

@@ -21,8 +21,9 @@ struct DevStatus {
 
 // Stage plan of a stage-planned SpMV configuration (stage.cu).
 struct StagePlan {
+    void *mem = nullptr;      // one allocation for the arrays below
     int32_t *part = nullptr;  // warps + 1 slice boundaries
-    int64_t *sptr = nullptr;  // warps + 1 starts of each warp's boundary list
+    int32_t *cnt = nullptr;   // stages of each warp
     int32_t *sb = nullptr;    // boundary lists (relative word offsets)
     int blocks = 0, warps = 0;
 };
@@ -50,7 +51,8 @@ struct Matrix {
     static constexpr int kBulkVariants = 3;
     int variant = 0;       // 0 auto, 1 thread-per-row, 2.. bulk-staged configs
     int auto_variant = 1;  // what variant 0 runs (set by the plan or the tuner)
-    int32_t *part[kBulkVariants] = {};  // part_warps + 1 slice boundaries
+    int32_t *part[kBulkVariants] = {};  // part_warps + 1 slice boundaries (one allocation, part_mem)
+    void *part_mem = nullptr;
     int part_warps[kBulkVariants] = {};
     int part_blocks[kBulkVariants] = {};
     static constexpr int kStageVariants = 2;  // variants 9, 10
@@ -98,7 +100,29 @@ packsell_status encode_impl(const packsell_params &p, int64_t n, int64_t m, int6
                             int val_is_f64, cudaStream_t s, Matrix **out);
 packsell_status validate_impl(const Matrix &A, cudaStream_t s, const char *what);
 void destroy_matrix(Matrix *A);
-packsell_status scan_i64(const int64_t *in, int64_t *out, int64_t S, cudaStream_t s);
+
+// pool.cu: stream-ordered device memory from the library's pool (one per
+// device). pool_get: usable by work on `s`, and by any stream once `s` has
+// been synchronised; pool_put: returned once the work already on `s` is done.
+cudaError_t pool_get(void **p, size_t bytes, cudaStream_t s);
+template <typename T>
+cudaError_t pool_get(T **p, size_t bytes, cudaStream_t s) {
+    return pool_get(reinterpret_cast<void **>(p), bytes, s);
+}
+void pool_put(void *p, cudaStream_t s);
+
+// How an object's arrays are given back: in the order of a stream (every use
+// of them lies before on that stream, or the device has been synchronised),
+// or by cudaFree, which waits for the device.
+struct Release {
+    bool ordered;
+    cudaStream_t s;
+    void operator()(void *p) const {
+        if (!p) return;
+        if (ordered) pool_put(p, s);
+        else cudaFree(p);
+    }
+};
 packsell_status quantize_impl(int fmt, int D, int64_t n, const void *val, int is64, uint32_t *field,
                               int64_t *bad_index, cudaStream_t s);
 // max_i sum_j |a_ij - q(a_ij)|, max_i sum_j |q(a_ij)|, max_i sum_j |a_ij| for a
@@ -110,7 +134,7 @@ packsell_status format_error_impl(int64_t n, const int64_t *rowptr, const void *
 
 // stage.cu
 packsell_status plan_stage(Matrix &A, cudaStream_t s);
-void stage_free(Matrix &A);
+void stage_free(Matrix &A, const Release &rel);
 
 // w16.cu
 packsell_status spmv_w16_impl(const Matrix &A, const float *x, float *y, cudaStream_t s);
@@ -120,7 +144,7 @@ packsell_status spmv_x16_impl(const Matrix &A, const uint16_t *x, uint16_t *y, c
 
 // csr.cu
 packsell_status plan_csr(Matrix &A, cudaStream_t s);
-void csr_plan_free(Matrix &A);
+void csr_plan_free(Matrix &A, const Release &rel);
 packsell_status launch_csr(const Matrix &A, const void *perm, int pb, const float *x, float *y,
                            cudaStream_t s);
 // multi.cu: split-row products with k right-hand sides over CSR-order
@@ -149,13 +173,13 @@ SplitMat split_mat(const Matrix &A, const float *X, int64_t ldx, float *Y, int64
 void multi_items_append(const int64_t *off, int64_t n, int mat, std::vector<MultiItem> &items);
 void multi_items_order(std::vector<MultiItem> &items);
 packsell_status multi_plan(Matrix &A, cudaStream_t s);
-void multi_plan_free(Matrix &A);
+void multi_plan_free(Matrix &A, const Release &rel);
 packsell_status launch_multi(const SplitMat &single, const SplitMat *mats, const MultiItem *items,
                              int nitems, int k, bool vec, cudaStream_t s);
 
 // split.cu
 packsell_status plan_split(Matrix &A, cudaStream_t s);
-void split_plan_free(Matrix &A);
+void split_plan_free(Matrix &A, const Release &rel);
 packsell_status split_items_append(const int64_t *off, int64_t n, int mat,
                                    std::vector<MultiItem> &items);
 packsell_status launch_split_batch(const SplitMat *mats, const MultiItem *items, int nitems,

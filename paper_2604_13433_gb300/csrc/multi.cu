@@ -791,14 +791,13 @@ void multi_items_order(std::vector<MultiItem> &items) {
                      [](const MultiItem &a, const MultiItem &b) { return a.meta < b.meta; });
 }
 
-void multi_plan_free(Matrix &A) {
-    cudaFree(A.multi_items);
+void multi_plan_free(Matrix &A, const Release &rel) {
+    rel(A.multi_items);
     A.multi_items = nullptr;
     A.multi_nitems = 0;
 }
 
 packsell_status multi_plan(Matrix &A, cudaStream_t s) {
-    multi_plan_free(A);
     if (!is_packed(A.p.format) || A.p.C != 1 || A.n == 0) return PACKSELL_OK;
     std::vector<int64_t> off((size_t)A.n + 1);
     PS_CUDA(cudaMemcpyAsync(off.data(), A.offset, sizeof(int64_t) * (A.n + 1),
@@ -809,9 +808,10 @@ packsell_status multi_plan(Matrix &A, cudaStream_t s) {
     multi_items_append(off.data(), A.n, 0, items);
     multi_items_order(items);
     if (items.size() >= (size_t)INT32_MAX) return fail(PACKSELL_ERR_RANGE, "multi_plan: too many items");
-    PS_CUDA(cudaMalloc(&A.multi_items, sizeof(MultiItem) * items.size()));
-    PS_CUDA(cudaMemcpy(A.multi_items, items.data(), sizeof(MultiItem) * items.size(),
-                       cudaMemcpyHostToDevice));
+    PS_CUDA(pool_get(&A.multi_items, sizeof(MultiItem) * items.size(), s));
+    PS_CUDA(cudaMemcpyAsync(A.multi_items, items.data(), sizeof(MultiItem) * items.size(),
+                            cudaMemcpyHostToDevice, s));
+    PS_CUDA(cudaStreamSynchronize(s));
     A.multi_nitems = (int)items.size();
     return PACKSELL_OK;
 }

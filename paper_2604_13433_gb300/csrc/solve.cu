@@ -431,7 +431,7 @@ packsell_status solve_impl(const Matrix *A64, const Matrix *Ain, const double *i
             st = fail(PACKSELL_ERR_INVALID_ARG, "packsell_pcg: no workspace");
             goto out;
         }
-        if (cudaMallocAsync(&own, need, s) != cudaSuccess) {
+        if (pool_get(&own, need, s) != cudaSuccess) {
             st = fail(PACKSELL_ERR_NO_MEMORY, "packsell_pcg: workspace allocation");
             goto out;
         }
@@ -598,7 +598,7 @@ packsell_status solve_impl(const Matrix *A64, const Matrix *Ain, const double *i
 out:
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
-    if (own) cudaFreeAsync(own, s);
+    if (own) pool_put(own, s);
     cudaStreamSynchronize(s);
     if (ev0) cudaEventDestroy(ev0);
     if (ev1) cudaEventDestroy(ev1);

@@ -657,8 +657,8 @@ int split_blocks() {
 
 }  // namespace
 
-void split_plan_free(Matrix &A) {
-    cudaFree(A.split_items);
+void split_plan_free(Matrix &A, const Release &rel) {
+    rel(A.split_items);
     A.split_items = nullptr;
     A.split_nitems = 0;
 }
@@ -700,7 +700,6 @@ static packsell_status split_cut(const int64_t *off, int n, Push push) {
 // row offsets by split_cut. Long rows come first, longest first: they are the
 // longest serial paths of the launch and start before the short tiles.
 packsell_status plan_split(Matrix &A, cudaStream_t s) {
-    split_plan_free(A);
     if (!is_packed(A.p.format) || A.p.C != 1 || A.n == 0) return PACKSELL_OK;
     std::vector<int64_t> off((size_t)A.n + 1);
     PS_CUDA(cudaMemcpyAsync(off.data(), A.offset, sizeof(int64_t) * (A.n + 1),
@@ -719,7 +718,7 @@ packsell_status plan_split(Matrix &A, cudaStream_t s) {
                      [](const SplitItem &a, const SplitItem &b) { return a.meta < b.meta; });
     if (items.size() >= (size_t)INT32_MAX)
         return fail(PACKSELL_ERR_RANGE, "plan_split: too many items");
-    PS_CUDA(cudaMalloc(&A.split_items, sizeof(SplitItem) * items.size()));
+    PS_CUDA(pool_get(&A.split_items, sizeof(SplitItem) * items.size(), s));
     PS_CUDA(cudaMemcpyAsync(A.split_items, items.data(), sizeof(SplitItem) * items.size(),
                             cudaMemcpyHostToDevice, s));
     PS_CUDA(cudaStreamSynchronize(s));

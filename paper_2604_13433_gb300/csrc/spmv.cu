@@ -729,11 +729,17 @@ PS_BULK_KERNEL(1, 4, 3, 512, 9, false)
 PS_BULK_KERNEL(2, 8, 2, 1024, 3, true)
 #undef PS_BULK_KERNEL
 
-// part[g] = first slice whose word offset reaches g * N_w / G, g = 0..G.
-__global__ void k_partition(int64_t S, const int64_t *__restrict__ offset, int G,
-                            int32_t *__restrict__ part) {
+// part[g] = first slice whose word offset reaches g * N_w / G, g = 0..G, for
+// each bulk configuration (blockIdx.y)
+struct PartArgs {
+    int32_t *part[Matrix::kBulkVariants];
+    int G[Matrix::kBulkVariants];  // 0: not planned
+};
+
+__global__ void k_partition(int64_t S, const int64_t *__restrict__ offset, PartArgs a) {
     int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g > G) return;
+    const int G = a.G[blockIdx.y];
+    if (G == 0 || g > G) return;
     int64_t total = offset[S];
     int64_t target = (int64_t)((__int128)total * g / G);
     int64_t lo = 0, hi = S;  // first k in [0, S] with offset[k] >= target
@@ -742,7 +748,7 @@ __global__ void k_partition(int64_t S, const int64_t *__restrict__ offset, int G
         if (offset[mid] >= target) hi = mid;
         else lo = mid + 1;
     }
-    part[g] = (int32_t)(g == G ? S : lo);
+    a.part[blockIdx.y][g] = (int32_t)(g == G ? S : lo);
 }
 
 template <int FMT>
@@ -752,6 +758,28 @@ void *bulk_fn(int v) {
         case 1: return (void *)BulkKernel<FMT, 1>::fn;
         default: return (void *)BulkKernel<FMT, 2>::fn;
     }
+}
+
+// Blocks of configuration v resident at once on the current device (its
+// shared-memory limit is raised on the first use; cached per device).
+template <int FMT>
+packsell_status bulk_grid(int v, int *blocks) {
+    static std::atomic<int> cached[64][Matrix::kBulkVariants];
+    int dev = 0;
+    PS_CUDA(cudaGetDevice(&dev));
+    int b = dev < 64 ? cached[dev][v].load(std::memory_order_relaxed) : 0;
+    if (!b) {
+        const BulkCfg &cf = kBulkCfg[v];
+        void *fn = bulk_fn<FMT>(v);
+        int sms = 0, per = 0;
+        PS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        PS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cf.smem()));
+        PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, cf.nw * 32, cf.smem()));
+        b = per < 1 ? -1 : sms * per;
+        if (dev < 64) cached[dev][v].store(b, std::memory_order_relaxed);
+    }
+    *blocks = b;
+    return PACKSELL_OK;
 }
 
 template <int FMT>
@@ -1031,7 +1059,7 @@ void set_data_wait_limit(uint32_t limit) { g_wait_limit.store(limit, std::memory
 // slice partition balanced by words. Variant 0 then runs configuration 0.
 packsell_status plan_spmv(Matrix &A, cudaStream_t s) {
     if (!A.status) {
-        PS_CUDA(cudaMalloc(&A.status, sizeof(DevStatus)));
+        PS_CUDA(pool_get(&A.status, sizeof(DevStatus), s));
         PS_CUDA(cudaMemsetAsync(A.status, 0, sizeof(DevStatus), s));
     }
     A.auto_variant = 1;
@@ -1053,25 +1081,31 @@ packsell_status plan_spmv(Matrix &A, cudaStream_t s) {
     // the bulk kernel indexes a warp's words with 32-bit integers
     if (!is_packed(A.p.format) || A.p.C != 32 || A.n == 0 || A.n_words >= (1ll << 31) - 4096)
         return PACKSELL_OK;
-    int dev = 0, sms = 0;
-    PS_CUDA(cudaGetDevice(&dev));
-    PS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    PartArgs pa{};
+    size_t entries = 0;
+    int most = 0;
     for (int v = 0; v < Matrix::kBulkVariants; ++v) {
-        const BulkCfg &cf = kBulkCfg[v];
-        void *fn = A.p.format == PACKSELL_FMT_FP16 ? bulk_fn<PACKSELL_FMT_FP16>(v)
-                                                   : bulk_fn<PACKSELL_FMT_E8MY>(v);
-        PS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cf.smem()));
-        int per_sm = 0;
-        PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, cf.nw * 32, cf.smem()));
-        if (per_sm < 1) continue;
-        const int blocks = sms * per_sm, G = blocks * cf.nw;
-        if (A.part[v]) cudaFree(A.part[v]);
-        A.part[v] = nullptr;
-        PS_CUDA(cudaMalloc(&A.part[v], sizeof(int32_t) * (G + 1)));
-        k_partition<<<(G + 1 + 255) / 256, 256, 0, s>>>(A.n_slices, A.offset, G, A.part[v]);
-        PS_LAUNCH_CHECK("k_partition");
+        int blocks = 0;
+        const packsell_status st = A.p.format == PACKSELL_FMT_FP16
+                                       ? bulk_grid<PACKSELL_FMT_FP16>(v, &blocks)
+                                       : bulk_grid<PACKSELL_FMT_E8MY>(v, &blocks);
+        if (st != PACKSELL_OK) return st;
+        if (blocks < 1) continue;
         A.part_blocks[v] = blocks;
-        A.part_warps[v] = G;
+        A.part_warps[v] = pa.G[v] = blocks * kBulkCfg[v].nw;
+        entries += pa.G[v] + 1;
+        most = std::max(most, pa.G[v]);
+    }
+    if (most > 0) {
+        PS_CUDA(pool_get(&A.part_mem, sizeof(int32_t) * entries, s));
+        int32_t *at = (int32_t *)A.part_mem;
+        for (int v = 0; v < Matrix::kBulkVariants; ++v) {
+            if (!pa.G[v]) continue;
+            A.part[v] = pa.part[v] = at;
+            at += pa.G[v] + 1;
+        }
+        k_partition<<<dim3((most + 256) / 256, Matrix::kBulkVariants), 256, 0, s>>>(A.n_slices, A.offset, pa);
+        PS_LAUNCH_CHECK("k_partition");
     }
     // untuned default (variant 0), by matrix shape: every slice within one
     // round -> the pipelined kernel; padding above 1/8 of the words (uneven

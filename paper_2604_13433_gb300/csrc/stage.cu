@@ -15,6 +15,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "device.cuh"
 #include "internal.h"
@@ -24,48 +25,70 @@ namespace {
 
 // ---- plan: stage boundaries per warp ----------------------------------------
 // Boundaries are word offsets relative to the warp's first word; warp g's
-// list sb[sptr[g] .. sptr[g+1]) holds (stages + 1) entries, 0 first, the
-// warp's word count last.
-template <bool FILL>
-__global__ void k_stage_plan(int G, const int32_t *__restrict__ part,
-                             const int64_t *__restrict__ offset, int SW,
-                             int64_t *__restrict__ count, const int64_t *__restrict__ sptr,
-                             int32_t *__restrict__ sb) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
-    const int k0 = part[g], k1 = part[g + 1];
-    const int64_t base = k0 < k1 ? offset[k0] : 0;
-    int64_t nb = 0;  // boundaries written after the leading 0
-    int32_t *out = FILL ? sb + sptr[g] : nullptr;
-    if (FILL) out[0] = 0;
-    auto emit = [&](int64_t b) {
-        ++nb;
-        if (FILL) out[nb] = (int32_t)b;
-    };
+// list holds (stages + 1) entries, 0 first, the warp's word count last. Two
+// adjacent stages hold more than SW words together, so a warp of w words has
+// at most 2 w / SW + 1 stages: its list starts at list_start(), where the
+// lists of the warps before it cannot reach, and the plan needs neither a
+// counting pass nor a read-back of its size.
+__device__ __forceinline__ int64_t list_start(int64_t first_word, int SW, int g) {
+    return 2 * first_word / SW + 4ll * g;
+}
+
+// first slice whose word offset reaches g * N_w / G
+__device__ __forceinline__ int32_t part_bound(int64_t S, const int64_t *__restrict__ offset, int g,
+                                              int G) {
+    if (g >= G) return (int32_t)S;
+    const int64_t target = (int64_t)((__int128)offset[S] * g / G);
+    int64_t lo = 0, hi = S;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (offset[mid] >= target) hi = mid;
+        else lo = mid + 1;
+    }
+    return (int32_t)lo;
+}
+
+struct StageArgs {
+    int32_t *part, *cnt, *sb;
+    int G, SW;
+};
+
+// Both configurations in one launch (blockIdx.y): partition and lists.
+__global__ void k_stage_plan(int64_t S, const int64_t *__restrict__ offset, StageArgs a0, StageArgs a1) {
+    const StageArgs a = blockIdx.y == 0 ? a0 : a1;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x, SW = a.SW;
+    if (g >= a.G) return;
+    const int k0 = part_bound(S, offset, g, a.G), k1 = part_bound(S, offset, g + 1, a.G);
+    a.part[g] = k0;
+    if (g == a.G - 1) a.part[a.G] = (int32_t)S;
+    const int64_t base = offset[k0];
+    int32_t *out = a.sb + list_start(base, SW, g);
+    int nb = 0;  // boundaries written after the leading 0
+    out[0] = 0;
     int64_t cur_lo = 0, cur_hi = 0;
     for (int k = k0; k < k1; ++k) {
         const int64_t lo = offset[k] - base, hi = offset[k + 1] - base;
         if (hi == lo) continue;
         if (hi - lo <= SW) {
             if (hi - cur_lo > SW) {
-                emit(lo);
+                out[++nb] = (int32_t)lo;
                 cur_lo = lo;
             }
             cur_hi = hi;
         } else {
             if (cur_hi > cur_lo) {
-                emit(lo);
+                out[++nb] = (int32_t)lo;
                 cur_lo = lo;
             }
             for (int64_t b = lo + SW; b < hi; b += SW) {
-                emit(b);
+                out[++nb] = (int32_t)b;
                 cur_lo = b;
             }
             cur_hi = hi;
         }
     }
-    if (cur_hi > cur_lo) emit(cur_hi);  // closes the last stage at the warp's word count
-    if (!FILL) count[g] = nb + 1;       // entries of the list
+    if (cur_hi > cur_lo) out[++nb] = (int32_t)cur_hi;  // closes the last stage at the warp's word count
+    a.cnt[g] = nb;
 }
 
 // ---- the kernel ---------------------------------------------------------------
@@ -93,7 +116,7 @@ __global__ void __launch_bounds__(NW * 32, MINB)
                  const int64_t *__restrict__ offset, const uint32_t *__restrict__ pack,
                  const void *__restrict__ perm, int perm_bytes, Decode dc,
                  const float *__restrict__ x, float *__restrict__ y,
-                 const int32_t *__restrict__ part, const int64_t *__restrict__ sptr,
+                 const int32_t *__restrict__ part, const int32_t *__restrict__ scnt,
                  const int32_t *__restrict__ sbnd, DevStatus *st, uint32_t wait_limit) {
     static_assert((NS & (NS - 1)) == 0, "NS: power of two");
     extern __shared__ __align__(128) uint32_t ring_all[];
@@ -106,8 +129,8 @@ __global__ void __launch_bounds__(NW * 32, MINB)
     uint64_t *bar = bars[warp];
     const int64_t base = offset[k0];
     const uint32_t *src = pack + base;
-    const int32_t *B = sbnd + sptr[gw];
-    const int nst = (int)(sptr[gw + 1] - sptr[gw]) - 1;
+    const int32_t *B = sbnd + list_start(base, SW, gw);
+    const int nst = scnt[gw];
     const uint64_t pol = policy_evict_first();
     if (lane == 0) {
         for (int q = 0; q < NS; ++q) mbar_init(&bar[q], 1);
@@ -218,67 +241,65 @@ void *stage_fn(int v) {
     return v == 0 ? (void *)StageKernel<FMT, 0>::fn : (void *)StageKernel<FMT, 1>::fn;
 }
 
-__global__ void k_stage_partition(int64_t S, const int64_t *__restrict__ offset, int G,
-                                  int32_t *__restrict__ part) {
-    int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g > G) return;
-    int64_t total = offset[S];
-    int64_t target = (int64_t)((__int128)total * g / G);
-    int64_t lo = 0, hi = S;
-    while (lo < hi) {
-        int64_t mid = (lo + hi) >> 1;
-        if (offset[mid] >= target) hi = mid;
-        else lo = mid + 1;
+// Blocks of configuration v resident at once on the current device (its
+// shared-memory limit is raised on the first use; cached per device).
+template <int FMT>
+packsell_status stage_grid(int v, int *blocks) {
+    static std::atomic<int> cached[64][2];
+    int dev = 0;
+    PS_CUDA(cudaGetDevice(&dev));
+    int b = dev < 64 ? cached[dev][v].load(std::memory_order_relaxed) : 0;
+    if (!b) {
+        const StageCfg &cf = kStageCfg[v];
+        void *fn = stage_fn<FMT>(v);
+        int sms = 0, per = 0;
+        PS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        PS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cf.smem()));
+        PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, cf.nw * 32, cf.smem()));
+        b = per < 1 ? -1 : sms * per;
+        if (dev < 64) cached[dev][v].store(b, std::memory_order_relaxed);
     }
-    part[g] = (int32_t)(g == G ? S : lo);
+    *blocks = b;
+    return PACKSELL_OK;
 }
 
 }  // namespace
 
-void stage_free(Matrix &A) {
+void stage_free(Matrix &A, const Release &rel) {
     for (int v = 0; v < Matrix::kStageVariants; ++v) {
-        cudaFree(A.stage[v].part);
-        cudaFree(A.stage[v].sptr);
-        cudaFree(A.stage[v].sb);
+        rel(A.stage[v].mem);
         A.stage[v] = StagePlan{};
     }
 }
 
 packsell_status plan_stage(Matrix &A, cudaStream_t s) {
-    stage_free(A);
     if (!is_packed(A.p.format) || A.p.C != 32 || A.n == 0 || A.n_words >= (1ll << 31) - 4096)
         return PACKSELL_OK;
-    int dev = 0, sms = 0;
-    PS_CUDA(cudaGetDevice(&dev));
-    PS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    StageArgs args[Matrix::kStageVariants] = {};
+    int most = 0;
     for (int v = 0; v < Matrix::kStageVariants; ++v) {
-        const StageCfg &cf = kStageCfg[v];
-        void *fn = A.p.format == PACKSELL_FMT_FP16 ? stage_fn<PACKSELL_FMT_FP16>(v)
-                                                   : stage_fn<PACKSELL_FMT_E8MY>(v);
-        PS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cf.smem()));
-        int per = 0;
-        PS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, cf.nw * 32, cf.smem()));
-        if (per < 1) continue;
+        int blocks = 0;
+        const packsell_status st = A.p.format == PACKSELL_FMT_FP16
+                                       ? stage_grid<PACKSELL_FMT_FP16>(v, &blocks)
+                                       : stage_grid<PACKSELL_FMT_E8MY>(v, &blocks);
+        if (st != PACKSELL_OK) return st;
+        if (blocks < 1) continue;
         StagePlan &P = A.stage[v];
-        P.blocks = sms * per;
-        const int G = P.blocks * cf.nw;
+        const int G = blocks * kStageCfg[v].nw, SW = kStageCfg[v].sw;
+        const size_t lists = (size_t)(2 * A.n_words / SW + 4ll * G + 8);
+        if (cudaError_t e = pool_get(&P.mem, sizeof(int32_t) * ((size_t)2 * G + 1 + lists), s))
+            return cuda_fail(e, "plan_stage: plan arrays");
+        P.blocks = blocks;
         P.warps = G;
-        int64_t *cnt = nullptr;
-        PS_CUDA(cudaMalloc(&P.part, sizeof(int32_t) * (G + 1)));
-        PS_CUDA(cudaMalloc(&P.sptr, sizeof(int64_t) * (G + 1)));
-        PS_CUDA(cudaMallocAsync(&cnt, sizeof(int64_t) * G, s));
-        k_stage_partition<<<(G + 256) / 256, 256, 0, s>>>(A.n_slices, A.offset, G, P.part);
-        k_stage_plan<false><<<(G + 255) / 256, 256, 0, s>>>(G, P.part, A.offset, cf.sw, cnt, nullptr, nullptr);
-        packsell_status e = scan_i64(cnt, P.sptr, G, s);
-        if (e != PACKSELL_OK) return e;
-        int64_t total = 0;
-        PS_CUDA(cudaMemcpyAsync(&total, P.sptr + G, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        PS_CUDA(cudaStreamSynchronize(s));
-        PS_CUDA(cudaMalloc(&P.sb, sizeof(int32_t) * std::max<int64_t>(total, 1)));
-        k_stage_plan<true><<<(G + 255) / 256, 256, 0, s>>>(G, P.part, A.offset, cf.sw, nullptr, P.sptr, P.sb);
-        PS_CUDA(cudaFreeAsync(cnt, s));
-        PS_LAUNCH_CHECK("plan_stage");
+        P.part = (int32_t *)P.mem;
+        P.cnt = P.part + G + 1;
+        P.sb = P.cnt + G;
+        args[v] = StageArgs{P.part, P.cnt, P.sb, G, SW};
+        most = std::max(most, G);
     }
+    if (most == 0) return PACKSELL_OK;
+    k_stage_plan<<<dim3((most + 255) / 256, 2), 256, 0, s>>>(A.n_slices, A.offset, args[0], args[1]);
+    PS_LAUNCH_CHECK("plan_stage");
     return PACKSELL_OK;
 }
 
@@ -293,12 +314,11 @@ packsell_status launch_stage(const Matrix &A, int v, const void *perm, int pb, c
     Decode dc = make_decode(A);
     const int64_t *offset = A.offset;
     const uint32_t *pack = A.pack;
-    const int32_t *part = P.part, *sb = P.sb;
-    const int64_t *sptr = P.sptr;
+    const int32_t *part = P.part, *sb = P.sb, *cnt = P.cnt;
     DevStatus *st = A.status;
     uint32_t wl = data_wait_limit();
     void *args[] = {&n, &sg, &sh, &kl, (void *)&offset, (void *)&pack, (void *)&perm, &pb, &dc,
-                    (void *)&x, (void *)&y, (void *)&part, (void *)&sptr, (void *)&sb, (void *)&st,
+                    (void *)&x, (void *)&y, (void *)&part, (void *)&cnt, (void *)&sb, (void *)&st,
                     &wl};
     void *fn = A.p.format == PACKSELL_FMT_FP16 ? stage_fn<PACKSELL_FMT_FP16>(v)
                                                : stage_fn<PACKSELL_FMT_E8MY>(v);
