@@ -54,18 +54,22 @@ __device__ __forceinline__ long long dummies_of(long long d, long long lim, int 
 }
 
 // One warp per 32 rows, whose nonzeros are one contiguous run: the lanes read
-// 128 columns at a time, coalesced, each lane following the row its elements
-// belong to. A thread per row read its columns a row length apart from its
-// neighbours', twice (check, then count): 90 us on the 27-point 97 x 96 x 95
-// matrix (23.4M nonzeros), where one coalesced reading takes 14 us.
+// 128 columns at a time, four consecutive ones each (16 bytes), and compare
+// each with the one before it. Lane l also holds row l's start: which of the
+// 128 elements start a row is the union of the rows' bits, and the dummies of
+// a row are the difference of the warp's running count at its start and at
+// the next row's, read from the chunk's prefix counts in shared memory; no
+// lane searches for the row of its element. A thread per row read its
+// columns a row length apart from its neighbours', twice (check, then
+// count), and sent two atomics per warp to two addresses (1.7 ns each, one
+// after another): 90 us on the 27-point 97 x 96 x 95 matrix (23.4M nonzeros).
 constexpr int SCAN_W = 8;  // warps per block
 
 __global__ void __launch_bounds__(SCAN_W * 32)
     k_scan_rows(int n, int64_t m, int64_t nnz, const int64_t *__restrict__ rowptr,
                 const int32_t *__restrict__ col, int D, int packed, int W,
                 int32_t *__restrict__ words, int32_t *__restrict__ first, EncodeInfo *info) {
-    __shared__ long long s_start[SCAN_W][33];
-    __shared__ int s_first[SCAN_W][32], s_cnt[SCAN_W][32];
+    __shared__ __align__(16) int s_pre[SCAN_W][128];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int64_t r0 = ((int64_t)blockIdx.x * SCAN_W + wl) * 32;
     if (r0 == 0 && lane == 0) {
@@ -83,60 +87,102 @@ __global__ void __launch_bounds__(SCAN_W * 32)
         return;
     }
     const long long base = __shfl_sync(0xffffffffu, a, 0), end = __shfl_sync(0xffffffffu, b, rows - 1);
-    s_start[wl][lane] = live ? a : end;
-    if (lane == 0) s_start[wl][32] = end;
-    s_first[wl][lane] = -1;
-    s_cnt[wl][lane] = 0;
-    __syncwarp();
-    const long long lim = 1ll << D;
-    int row = 0, carry = 0;
-    for (long long p = base; p < end; p += 128) {
-        int c[4];
+    const bool filled = b > a;
+    const int f = filled ? __ldg(col + a) : -1;  // this lane's row's first column
+    const bool can_dummy = packed && D < 31;
+    int carry = 0;
+    long long run = 0, at_start = -1;  // dummies so far; before this lane's row (-1: not reached)
+    auto load = [&](long long e0, int (&c)[4]) {
+        c[0] = c[1] = c[2] = c[3] = 0;
+        if (e0 >= base && e0 + 4 <= end) {
+            const int4 q = __ldg(reinterpret_cast<const int4 *>(col + e0));
+            c[0] = q.x; c[1] = q.y; c[2] = q.z; c[3] = q.w;
+        } else {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const long long e = p + 32 * u + lane;
-            c[u] = e < end ? __ldg(col + e) : 0;
+            for (int j = 0; j < 4; ++j)
+                if (e0 + j >= base && e0 + j < end) c[j] = __ldg(col + e0 + j);
         }
+    };
+    // chunks start on 16-byte boundaries of the column array; the next chunk
+    // loads while this one is looked at
+    const long long p_first = base - (((uintptr_t)(col + base) >> 2) & 3);
+    int nxt[4];
+    load(p_first + 4 * lane, nxt);
+    for (long long p = p_first; p < end; p += 128) {
+        const long long e0 = p + 4 * lane;
+        const int c[4] = {nxt[0], nxt[1], nxt[2], nxt[3]};
+        load(e0 + 128, nxt);
+        // this lane's row start in the chunk, and the four bits of this lane's elements
+        const long long dl = a - p;
+        const int ds = filled && dl >= 0 && dl < 128 ? (int)dl : -1;
+        unsigned starts = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const long long e = p + 32 * u + lane;
-            int up = __shfl_up_sync(0xffffffffu, c[u], 1);
-            if (lane == 0) up = carry;
-            carry = __shfl_sync(0xffffffffu, c[u], 31);
-            int err = 0;
-            if (e < end) {
-                while (s_start[wl][row + 1] <= e) ++row;
-                if (c[u] < 0 || (int64_t)c[u] >= m) {
-                    err = PACKSELL_ERR_RANGE;
-                } else if (e == s_start[wl][row]) {
-                    s_first[wl][row] = c[u];
-                } else if (c[u] <= up && up < m) {  // an out-of-range column before it is the error
-                    err = PACKSELL_ERR_UNSORTED;
-                } else if (packed) {
-                    const long long nd = dummies_of((long long)c[u] - up, lim, W);
-                    if (nd) atomicAdd(&s_cnt[wl][row], (int)nd);
+            const unsigned mu = __reduce_or_sync(0xffffffffu, (ds >> 5) == u ? 1u << (ds & 31) : 0u);
+            if ((lane >> 3) == u) starts = mu >> (4 * (lane & 7));
+        }
+        int up = __shfl_up_sync(0xffffffffu, c[3], 1);
+        if (lane == 0) up = carry;
+        carry = __shfl_sync(0xffffffffu, c[3], 31);
+        int err = 0, ej = 0, nd[4];
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            nd[j] = 0;
+            if (e0 + j >= base && e0 + j < end) {
+                const bool st = (starts >> j) & 1u;
+                if ((unsigned)c[j] >= (unsigned)m) {  // (m < 2^31)
+                    if (!err) err = PACKSELL_ERR_RANGE, ej = j;
+                } else if (!st && c[j] <= up && up < m) {  // an out-of-range column before it is the error
+                    if (!err) err = PACKSELL_ERR_UNSORTED, ej = j;
+                } else if (!st && can_dummy && ((unsigned)(c[j] - up) >> D)) {
+                    nd[j] = (int)dummies_of((unsigned)(c[j] - up), 1ll << D, W);
+                    any = true;
                 }
             }
-            const unsigned mask = __ballot_sync(0xffffffffu, err != 0);
-            if (mask) {  // the first bad element of the warp's rows
-                if (lane == __ffs((int)mask) - 1) dev_fail(&info->st, err, e);
-                return;
+            up = c[j];
+        }
+        const unsigned em = __ballot_sync(0xffffffffu, err != 0);
+        if (em) {  // the first bad element of the warp's rows
+            if (lane == __ffs((int)em) - 1) dev_fail(&info->st, err, e0 + ej);
+            return;
+        }
+        if (__any_sync(0xffffffffu, any)) {
+            const int sum = nd[0] + nd[1] + nd[2] + nd[3];
+            int inc = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += v;
             }
+            const int pre = inc - sum;
+            reinterpret_cast<int4 *>(s_pre[wl])[lane] =
+                make_int4(pre, pre + nd[0], pre + nd[0] + nd[1], pre + nd[0] + nd[1] + nd[2]);
+            __syncwarp();
+            if (ds >= 0) at_start = run + s_pre[wl][ds];
+            __syncwarp();
+            run += __shfl_sync(0xffffffffu, inc, 31);
+        } else if (ds >= 0) {
+            at_start = run;
         }
     }
-    __syncwarp();
+    // a row's dummies: from its start to the next filled row's
+    if (!filled) at_start = run;
+    const unsigned fl = __ballot_sync(0xffffffffu, filled) & (lane == 31 ? 0u : 0xffffffffu << (lane + 1));
+    long long next = __shfl_sync(0xffffffffu, at_start, fl ? __ffs((int)fl) - 1 : lane);
+    if (!fl) next = run;
     unsigned dmax = 0;  // this row's i - (first column), if positive
     if (live) {
-        const long long cnt = b - a + s_cnt[wl][lane];
+        const long long cnt = b - a + (filled ? next - at_start : 0);
         if (cnt > 0x7fffffffll) dev_fail(&info->st, PACKSELL_ERR_RANGE, i);
         words[i] = (int32_t)cnt;
-        const int f = s_first[wl][lane];
         first[i] = f;
-        if (b > a && i > f) dmax = (unsigned)(i - f);
+        if (filled && i > f) dmax = (unsigned)(i - f);
     }
-    // one atomic per warp: millions of atomics on one address serialise
+    // only a warp that still raises the maximum sends an atomic
     dmax = __reduce_max_sync(0xffffffffu, dmax);
-    if (lane == 0 && dmax) atomicMax(&info->kl, (unsigned long long)dmax);
+    if (lane == 0 && dmax > *(volatile unsigned long long *)&info->kl)
+        atomicMax(&info->kl, (unsigned long long)dmax);
 }
 
 // FP16 value field: binary16 in bits 16..31, round to nearest even.
@@ -271,15 +317,17 @@ __global__ void k_quantize64(int64_t nnz, const T *__restrict__ val, int D,
 }
 
 // A word's value field for the formats of 32-bit words, as it is scattered.
-template <typename T>
-__device__ __forceinline__ int field32(int fmt, T v, int D, int s, uint32_t &f) {
-    return fmt == PACKSELL_FMT_FP16 ? field_fp16(v, f)
-           : fmt == PACKSELL_FMT_FIXED ? field_fixed(v, D, s, f)
+template <int FMT, typename T>
+__device__ __forceinline__ int field32(T v, int D, int s, uint32_t &f) {
+    return FMT == PACKSELL_FMT_FP16    ? field_fp16(v, f)
+           : FMT == PACKSELL_FMT_FIXED ? field_fixed(v, D, s, f)
                                        : field_e8my(v, D, f);
 }
 
 // The dummies of each row's first nonzero, whose delta (Eq. 4) needs k_left;
 // the total of the words and the longest row.
+constexpr int FIN_ROWS = 4;  // rows per thread: fewer blocks, fewer atomics on the totals
+
 __global__ void __launch_bounds__(TPB)
     k_finish_words(int n, const int64_t *__restrict__ rowptr, const int32_t *__restrict__ first,
                    int sigma, long long k_left_user, int D, int packed, int W,
@@ -292,10 +340,14 @@ __global__ void __launch_bounds__(TPB)
         s_max = 0;
     }
     __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    long long cnt = 0;
-    if (i < n) {
-        cnt = words[i];
+    unsigned long long v = 0;
+    int longest = 0;
+#pragma unroll
+    for (int u = 0; u < FIN_ROWS; ++u) {
+        const int64_t ii = ((int64_t)blockIdx.x * FIN_ROWS + u) * TPB + threadIdx.x;
+        if (ii >= n) break;
+        const int i = (int)ii;
+        long long cnt = words[i];
         const int f = first[i];
         if (packed && f >= 0) {
             const long long kl = k_left_user >= 0 ? k_left_user : (long long)info->kl;
@@ -311,9 +363,10 @@ __global__ void __launch_bounds__(TPB)
                 words[i] = (int32_t)cnt;
             }
         }
+        v += (unsigned long long)cnt;
+        longest = max(longest, (int)cnt);
     }
-    const int wmax = __reduce_max_sync(0xffffffffu, (int)cnt);
-    unsigned long long v = (unsigned long long)cnt;
+    const int wmax = __reduce_max_sync(0xffffffffu, longest);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(&s_total, v);
@@ -322,7 +375,7 @@ __global__ void __launch_bounds__(TPB)
     __syncthreads();
     if (threadIdx.x == 0 && s_max) {
         atomicAdd(&info->total, s_total);
-        atomicMax(&info->max_words, s_max);
+        if (s_max > *(volatile int *)&info->max_words) atomicMax(&info->max_words, s_max);
     }
 }
 
@@ -475,7 +528,7 @@ packsell_status scan_exclusive(const int64_t *in, int64_t *out, int64_t S, cudaS
         return PACKSELL_OK;
     }
     const int64_t B = (S + SCAN_CHUNK - 1) / SCAN_CHUNK;
-    if (B <= 8) {  // one block in up to eight trips costs no more than three launches
+    if (B <= 2) {  // a trip of one block takes 3.5 us, two more launches about 7
         k_scan_apply<<<1, SCAN_TPB, 0, s>>>(S, in, nullptr, out, total_out);
         PS_LAUNCH_CHECK("k_scan_apply");
         return PACKSELL_OK;
@@ -494,115 +547,126 @@ packsell_status scan_exclusive(const int64_t *in, int64_t *out, int64_t S, cudaS
 
 // Scatter into the column-major slice layout: word j of storage row i sits at
 // offset[k] + j*C + l (k = i / C, l = i % C). One warp per 32 storage rows, a
-// lane per row: the rows' columns and values come in rounds of 16 per row
-// through shared memory, half a warp reading each row's run of consecutive
-// entries (a lane walking its own row reads entries a row length apart from
-// its neighbours'), are quantised there, and the lanes' words of one j go out
-// together. Quantising here instead of in a pass of its own saves writing and
-// reading the fields: 59 + 69 us for the two passes on the 27-point
-// 97 x 96 x 95 matrix (23.4M nonzeros, 281 MB in and out).
+// lane per row: the rows' columns and values come in rounds of R per row into
+// shared memory (cp.async: no registers hold what is in flight), R lanes
+// reading each row's run of consecutive entries (a lane walking its own row
+// reads entries a row length apart from its neighbours'), are quantised
+// there, and the lanes' words of one j go out together. Quantising here
+// instead of in a pass of its own saves writing and reading the fields: 59 +
+// 69 us for the two passes on the 27-point 97 x 96 x 95 matrix (23.4M
+// nonzeros, 281 MB in and out). Rounds of 32 entries; of 8 where the rows
+// have no more on average (fewer idle lanes per copy).
 // Rows past n (phantom rows of the last slice) get padding only.
-constexpr int SC_W = 4;            // warps per block
-constexpr int SC_R = 16;           // entries of a row per round
-constexpr int SC_LD = SC_R + 1;    // staging stride (no bank conflicts between rows)
+constexpr int SC_W = 4;  // warps per block
 
 struct __align__(16) EntryRun {
     long long q;
     int cnt, pad;
 };
 
-template <typename T>
+template <int BYTES>
+__device__ __forceinline__ void cp_async_ca(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src), "n"(BYTES)
+                 : "memory");
+}
+
+template <typename T, int FMT, bool C32, int R>
 __global__ void __launch_bounds__(SC_W * 32)
-    k_scatter_packed(int n, int64_t rows_total, int C, int sigma, long long k_left, int fmt, int D,
+    k_scatter_packed(int n, int64_t rows_total, int Cr, int sigma, long long k_left, int D,
                      int value_exp, const int64_t *__restrict__ rowptr,
                      const int32_t *__restrict__ col, const T *__restrict__ val, const void *perm,
                      int perm_bytes, const int64_t *__restrict__ offset, uint32_t *__restrict__ pack,
                      DevStatus *st) {
-    __shared__ int32_t s_col[SC_W][32 * SC_LD];
-    __shared__ T s_val[SC_W][32 * SC_LD];
+    constexpr int LD = R + 1;  // staging stride (no bank conflicts between rows)
+    __shared__ int32_t s_col[SC_W][32 * LD];
+    __shared__ __align__(8) T s_val[SC_W][32 * LD];
     __shared__ EntryRun s_run[SC_W][32];
+    const int C = C32 ? 32 : Cr;
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int64_t ii = ((int64_t)blockIdx.x * SC_W + wl) * 32 + lane;
     if (ii - lane >= rows_total) return;  // warp-uniform
-    int64_t s = 0, w = 0;
-    int l = 0;
-    if (ii < rows_total) {
-        const int64_t k = ii / C;
-        l = (int)(ii - k * C);
-        s = offset[k];
-        w = (offset[k + 1] - s) / C;
-    }
-    uint32_t *dst = pack + s + l;
-    long long q = 0, prev = 0;
-    int len = 0;
+    long long q = 0;
+    int prev = 0, len = 0;
     if (ii < n) {
         const int r = orig_row((int)ii, sigma, perm, perm_bytes);
         q = rowptr[r];
         len = (int)(rowptr[r + 1] - q);
         prev = left_offset((int)ii, sigma, k_left);
     }
-    const long long lim = 1ll << D;
-    const int most = __reduce_max_sync(0xffffffffu, len), sub = lane & (SC_R - 1);
-    int64_t j = 0;
-    for (int t0 = 0; t0 < most; t0 += SC_R) {
-        const int here = max(0, min(SC_R, len - t0));
+    uint32_t *dst = pack, *dend = pack;
+    if (ii < rows_total) {
+        const int64_t k = ii / C, s = offset[k];
+        const int l = (int)(ii - k * C);
+        dst = pack + s + l;
+        dend = pack + offset[k + 1] + l;
+    }
+    const int most = __reduce_max_sync(0xffffffffu, len), sub = lane % R;
+    const int32_t *my_col = s_col[wl] + lane * LD;
+    const T *my_val = s_val[wl] + lane * LD;
+    for (int t0 = 0; t0 < most; t0 += R) {
+        const int here = max(0, min(R, len - t0));
         s_run[wl][lane] = EntryRun{q + t0, here, 0};
         __syncwarp();
 #pragma unroll 8
-        for (int k = 0; k < 16; ++k) {
-            const int r = 2 * k + (lane >> 4);
+        for (int k = 0; k < R; ++k) {
+            const int r = (32 / R) * k + lane / R;
             const EntryRun run = s_run[wl][r];
             if (sub < run.cnt) {
-                s_col[wl][r * SC_LD + sub] = __ldcs(col + run.q + sub);
-                s_val[wl][r * SC_LD + sub] = __ldcs(val + run.q + sub);
+                cp_async_ca<4>(&s_col[wl][r * LD + sub], col + run.q + sub);
+                cp_async_ca<(int)sizeof(T)>(&s_val[wl][r * LD + sub], val + run.q + sub);
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
-#pragma unroll 4
-        for (int u = 0; u < SC_R; ++u) {
-            if (u >= here) break;
-            const int c = s_col[wl][lane * SC_LD + u];
-            uint32_t f = 0;
-            const int err = field32(fmt, s_val[wl][lane * SC_LD + u], D, value_exp, f);
-            if (err) dev_fail(st, err, q + t0 + u);
-            long long d = c - prev;
-            if (d >= lim) {
-                dst[j * C] = (uint32_t)d << 1;  // dummy: flag 0, 31-bit delta
-                ++j;
-                d = 0;
+#pragma unroll 8
+        for (int u = 0; u < R; ++u) {
+            if (u < here) {
+                const int c = my_col[u];
+                uint32_t f = 0;
+                const int err = field32<FMT>(my_val[u], D, value_exp, f);
+                if (err) dev_fail(st, err, q + t0 + u);
+                uint32_t d = (uint32_t)(c - prev);
+                prev = c;
+                if (d >> D) {
+                    *dst = d << 1;  // dummy: flag 0, 31-bit delta
+                    dst += C;
+                    d = 0;
+                }
+                *dst = f | (d << 1) | 1u;
+                dst += C;
             }
-            dst[j * C] = f | ((uint32_t)d << 1) | 1u;
-            ++j;
-            prev = c;
         }
         __syncwarp();
     }
-    for (; j < w; ++j) dst[j * C] = 0u;
+    for (; dst < dend; dst += C) *dst = 0u;
 }
 
 // The same for CSR order (C = 1, sigma = 1): the words lie in the order of
 // the nonzeros, each nonzero after its dummy, so a warp takes the run of 32
 // rows 128 nonzeros at a time, coalesced in and out, with the dummies so far
 // as the shift between the two. Rows of any length cost the same.
-template <typename T>
+// bit e - p0 of each row start `a` that lies in [p0, p0 + 32) (none for an empty row)
+__device__ __forceinline__ unsigned start_bits(long long a, bool filled, long long p0) {
+    const long long d = a - p0;
+    return __reduce_or_sync(0xffffffffu, filled && d >= 0 && d < 32 ? 1u << (int)d : 0u);
+}
+
+template <typename T, int FMT>
 __global__ void __launch_bounds__(SCAN_W * 32)
-    k_scatter_csr(int n, long long k_left, int fmt, int D, int value_exp,
-                  const int64_t *__restrict__ rowptr, const int32_t *__restrict__ col,
-                  const T *__restrict__ val, const int64_t *__restrict__ offset,
-                  uint32_t *__restrict__ pack, DevStatus *st) {
-    __shared__ long long s_start[SCAN_W][33];
+    k_scatter_csr(int n, long long k_left, int D, int value_exp, const int64_t *__restrict__ rowptr,
+                  const int32_t *__restrict__ col, const T *__restrict__ val,
+                  const int64_t *__restrict__ offset, uint32_t *__restrict__ pack, DevStatus *st) {
+    __shared__ int s_left[SCAN_W][32];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int64_t r0 = ((int64_t)blockIdx.x * SCAN_W + wl) * 32;
     if (r0 >= n) return;
     const int rows = n - r0 < 32 ? (int)(n - r0) : 32;
     const long long base = rowptr[r0], end = rowptr[r0 + rows];
-    s_start[wl][lane] = lane < rows ? rowptr[r0 + lane] : end;
-    if (lane == 0) s_start[wl][32] = end;
-    __syncwarp();
-    const long long lim = 1ll << D;
+    const bool live = lane < rows;
+    const long long a = live ? rowptr[r0 + lane] : end, b = live ? rowptr[r0 + lane + 1] : end;
+    const int left = (int)max((long long)(r0 + lane) - k_left, 0ll);
     uint32_t *dst = pack + (offset[r0] - base);  // word of nonzero e, without dummies: dst[e]
-    int row = 0, carry = 0;
-    long long shift = 0;  // dummies so far
+    int carry = 0;
     for (long long p = base; p < end; p += 128) {
         int c[4];
         T v[4];
@@ -614,29 +678,32 @@ __global__ void __launch_bounds__(SCAN_W * 32)
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const long long e = p + 32 * u + lane;
+            const long long p0 = p + 32 * u, e = p0 + lane;
+            if (p0 >= end) break;  // warp-uniform
             int up = __shfl_up_sync(0xffffffffu, c[u], 1);
             if (lane == 0) up = carry;
             carry = __shfl_sync(0xffffffffu, c[u], 31);
-            long long d = 0;
-            if (e < end) {
-                while (s_start[wl][row + 1] <= e) ++row;
-                const long long left = max((long long)(r0 + row) - k_left, 0ll);
-                d = c[u] - (e == s_start[wl][row] ? left : (long long)up);
+            const unsigned sb = start_bits(a, b > a, p0);
+            if (sb) {  // a row's first delta is taken from its left offset
+                if (b > a && a >= p0 && a < p0 + 32) s_left[wl][(int)(a - p0)] = left;
+                __syncwarp();
+                if ((sb >> lane) & 1u) up = s_left[wl][lane];
+                __syncwarp();
             }
-            const unsigned dm = __ballot_sync(0xffffffffu, d >= lim);
+            uint32_t d = e < end ? (uint32_t)(c[u] - up) : 0u;
+            const unsigned dm = __ballot_sync(0xffffffffu, (d >> D) != 0u);
             if (e < end) {
                 uint32_t f = 0;
-                const int err = field32(fmt, v[u], D, value_exp, f);
+                const int err = field32<FMT>(v[u], D, value_exp, f);
                 if (err) dev_fail(st, err, e);
-                uint32_t *at = dst + e + shift + __popc(dm & (0xffffffffu >> (31 - lane)));
-                if (d >= lim) {
-                    at[-1] = (uint32_t)d << 1;
+                uint32_t *at = dst + e + __popc(dm & (0xffffffffu >> (31 - lane)));
+                if (d >> D) {
+                    at[-1] = d << 1;
                     d = 0;
                 }
-                *at = f | ((uint32_t)d << 1) | 1u;
+                *at = f | (d << 1) | 1u;
             }
-            shift += __popc(dm);
+            dst += __popc(dm);  // the dummies so far
         }
     }
 }
@@ -939,7 +1006,7 @@ packsell_status encode_impl(const packsell_params &p, int64_t n, int64_t m, int6
                                                      A->value_exp);
         }
         if (n > 0) {
-            k_finish_words<<<blocks_for(n), TPB, 0, s>>>((int)n, rowptr, first, p.sigma, p.k_left, D,
+            k_finish_words<<<blocks_for(n, TPB * FIN_ROWS), TPB, 0, s>>>((int)n, rowptr, first, p.sigma, p.k_left, D,
                                                         packed ? 1 : 0, W, words, info);
             if (sorted) {
                 int64_t nb = (n + p.sigma - 1) / p.sigma;
@@ -1001,19 +1068,32 @@ packsell_status encode_impl(const packsell_params &p, int64_t n, int64_t m, int6
             if (pool_get(&A->pack, sizeof(uint32_t) * (nw + kWordTail), s) != cudaSuccess)
                 return bail(fail(PACKSELL_ERR_NO_MEMORY, "packsell_encode: word array"));
             int64_t rows_total = S * p.C;
-            auto scatter = [&](auto *v) {
+            auto scatter = [&](auto *v, auto format) {
                 using T = std::remove_const_t<std::remove_pointer_t<decltype(v)>>;
-                if (p.C == 1 && !sorted)
-                    k_scatter_csr<T><<<blocks_for(n, SCAN_W * 32), SCAN_W * 32, 0, s>>>(
-                        (int)n, A->p.k_left, fmt, D, A->value_exp, rowptr, col, v, A->offset, A->pack, st);
+                constexpr int F = decltype(format)::value;
+                if (p.C == 1 && !sorted) {
+                    k_scatter_csr<T, F><<<blocks_for(n, SCAN_W * 32), SCAN_W * 32, 0, s>>>(
+                        (int)n, A->p.k_left, D, A->value_exp, rowptr, col, v, A->offset, A->pack, st);
+                    return;
+                }
+                const bool few = nnz <= 8 * n;  // entries per row on average
+                auto k = p.C == 32 ? (few ? k_scatter_packed<T, F, true, 8> : k_scatter_packed<T, F, true, 32>)
+                                   : (few ? k_scatter_packed<T, F, false, 8> : k_scatter_packed<T, F, false, 32>);
+                k<<<blocks_for(rows_total, SC_W * 32), SC_W * 32, 0, s>>>(
+                    (int)n, rows_total, p.C, p.sigma, A->p.k_left, D, A->value_exp, rowptr, col, v,
+                    A->perm, perm_bytes, A->offset, A->pack, st);
+            };
+            auto scatter_fmt = [&](auto *v) {
+                if (fmt == PACKSELL_FMT_FP16)
+                    scatter(v, std::integral_constant<int, PACKSELL_FMT_FP16>());
+                else if (is_fixed(fmt))
+                    scatter(v, std::integral_constant<int, PACKSELL_FMT_FIXED>());
                 else
-                    k_scatter_packed<T><<<blocks_for(rows_total, SC_W * 32), SC_W * 32, 0, s>>>(
-                        (int)n, rows_total, p.C, p.sigma, A->p.k_left, fmt, D, A->value_exp, rowptr,
-                        col, v, A->perm, perm_bytes, A->offset, A->pack, st);
+                    scatter(v, std::integral_constant<int, PACKSELL_FMT_E8MY>());
             };
             if (rows_total > 0) {
-                if (val_is_f64) scatter((const double *)val);
-                else scatter((const float *)val);
+                if (val_is_f64) scatter_fmt((const double *)val);
+                else scatter_fmt((const float *)val);
             }
         } else if (is_sell16(fmt)) {
             if (pool_get(&A->val, 2 * std::max<int64_t>(nw, 1), s) != cudaSuccess ||
