@@ -178,9 +178,7 @@ __global__ void __launch_bounds__(FT) k_scale(int64_t n, const TI *__restrict__ 
 
 // h[j+1][j] = ||w||; the earlier Givens rotations on column j, a new one
 // that zeroes h[j+1][j]; g updated; scal[1] = 1 / h[j+1][j], scal[2] = |g[j+1]|
-__device__ __forceinline__ void arnoldi_finish(int G, const double *part, Hess h, int j, double *sh) {
-    const double s = partial_sum(part, G, sh);
-    if (threadIdx.x != 0) return;
+__device__ __forceinline__ void givens_column(double s, Hess h, int j) {  // s = w.w
     const int ld = h.m + 1;
     double *col = h.H + (int64_t)j * ld;
     const double hn = sqrt(s);
@@ -201,6 +199,11 @@ __device__ __forceinline__ void arnoldi_finish(int G, const double *part, Hess h
     h.g[j] = c * h.g[j];
     h.scal[1] = hn > 0.0 ? 1.0 / hn : 0.0;
     h.scal[2] = fabs(h.g[j + 1]);
+}
+
+__device__ __forceinline__ void arnoldi_finish(int G, const double *part, Hess h, int j, double *sh) {
+    const double s = partial_sum(part, G, sh);
+    if (threadIdx.x == 0) givens_column(s, h, j);
 }
 
 // w = w - sum_i h[i][j] v_i (in double, rounded once to T); partials of w.w;
@@ -239,6 +242,168 @@ __global__ void __launch_bounds__(FT) k_orth(int64_t n, const T *__restrict__ V,
     s = block_sum(s, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = s;
     if (last_block(counter)) arnoldi_finish(gridDim.x, part, h, j, sh);
+}
+
+// ---- an Arnoldi step's vector work in one kernel (FP32 layers) ----
+// The three kernels above read the new vector w three times and write it
+// twice, and each ends in a reduction that the next one waits for: on the
+// 27-point 128^3 matrix (8.4 MB vectors, all in L2) a step of layer 3 spent
+// about 50 us in them (F3R 64.5 ms; 62.4 ms with this kernel, 56.4 ms with the
+// Richardson steps in the products' epilogues as well). Here every thread keeps its E elements of w in
+// registers through the dot products, the update and the scaling, and the
+// blocks (all resident: a cooperative launch) meet twice. Every block adds
+// all partials itself, in block order, so all have the same sums.
+struct Meet {
+    unsigned *arrived, *left;  // 0 between launches
+    int *timeout;              // set when a wait ran out: later launches return at once
+};
+
+constexpr unsigned kMeetPolls = 1u << 22;
+
+// Wait (bounded) until all blocks have arrived `round` times; false when the wait ran out.
+__device__ __forceinline__ bool meet(const Meet &m, unsigned round) {
+    __shared__ bool ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(m.arrived, 1u);
+        const unsigned all = gridDim.x * round;
+        unsigned polls = 0;
+        while (*(volatile unsigned *)m.arrived < all && ++polls < kMeetPolls) __nanosleep(32);
+        ok = polls < kMeetPolls;
+        if (!ok) *m.timeout = 1;
+        __threadfence();
+    }
+    __syncthreads();
+    return ok;
+}
+
+// The last block to call this after the last meet() puts the counters back.
+__device__ __forceinline__ void meet_done(const Meet &m) {
+    if (threadIdx.x == 0 && atomicAdd(m.left, 1u) == gridDim.x - 1u) {
+        *m.arrived = 0u;
+        *m.left = 0u;
+    }
+}
+
+template <int E>
+__global__ void __launch_bounds__(FT, 4)
+    k_arnoldi(int64_t n, const float *__restrict__ V, int cnt, Hess h, int j, float *__restrict__ w,
+              double *__restrict__ part, Meet m) {
+    __shared__ double sh[64][FT / 32];
+    __shared__ float hf[64];
+    __shared__ double s_norm;
+    if (*(volatile int *)m.timeout) return;
+    const int G = gridDim.x, wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t tid = blockIdx.x * (int64_t)FT + threadIdx.x, st = (int64_t)G * FT, nv = n / 4;
+    float4 a[E / 4];
+#pragma unroll
+    for (int k = 0; k < E / 4; ++k) {
+        const int64_t v = tid + k * st;
+        a[k] = v < nv ? reinterpret_cast<const float4 *>(w)[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    // the n % 4 elements after the last whole vector, one thread each
+    const int64_t te = nv * 4 + tid;
+    const bool tail = te < n;
+    float at = tail ? w[te] : 0.f;
+    // the lanes' sums of one quantity into sh[i][warp]
+    auto publish = [&](int i, float f) {
+        double d = (double)f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane == 0) sh[i][wl] = d;
+    };
+    // the grid's sum of one quantity, every lane of the warp (partials in block order)
+    auto total = [&](const double *p) {
+        double s = 0.0;
+        for (int b = lane; b < G; b += 32) s += ((const volatile double *)p)[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    };
+    auto block_parts = [&](int count, double *out) {  // sh -> one partial per block and quantity
+        __syncthreads();
+        for (int i = threadIdx.x; i < count; i += FT) {
+            double s = 0.0;
+#pragma unroll
+            for (int q = 0; q < FT / 32; ++q) s += sh[i][q];
+            out[(int64_t)i * G + blockIdx.x] = s;
+        }
+    };
+    for (int i = 0; i < cnt; ++i) {
+        const float *__restrict__ v = V + (int64_t)i * n;
+        const bool al = ((uintptr_t)v & 15u) == 0;
+        float f = tail ? at * v[te] : 0.f;
+#pragma unroll
+        for (int k = 0; k < E / 4; ++k) {
+            const int64_t q = tid + k * st;
+            if (q < nv) {
+                const float4 b = al ? reinterpret_cast<const float4 *>(v)[q]
+                                    : make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                f = fmaf(a[k].x, b.x, f);
+                f = fmaf(a[k].y, b.y, f);
+                f = fmaf(a[k].z, b.z, f);
+                f = fmaf(a[k].w, b.w, f);
+            }
+        }
+        publish(i, f);
+    }
+    block_parts(cnt, part);
+    if (!meet(m, 1)) return;
+    for (int i = wl; i < cnt; i += FT / 32) {
+        const double s = total(part + (int64_t)i * G);
+        if (lane == 0) {
+            hf[i] = (float)s;
+            if (blockIdx.x == 0) h.H[i + (int64_t)j * (h.m + 1)] = s;
+        }
+    }
+    __syncthreads();
+    for (int i = 0; i < cnt; ++i) {
+        const float *__restrict__ v = V + (int64_t)i * n;
+        const bool al = ((uintptr_t)v & 15u) == 0;
+        const float c = -hf[i];
+        if (tail) at = fmaf(c, v[te], at);
+#pragma unroll
+        for (int k = 0; k < E / 4; ++k) {
+            const int64_t q = tid + k * st;
+            if (q < nv) {
+                const float4 b = al ? reinterpret_cast<const float4 *>(v)[q]
+                                    : make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                a[k].x = fmaf(c, b.x, a[k].x);
+                a[k].y = fmaf(c, b.y, a[k].y);
+                a[k].z = fmaf(c, b.z, a[k].z);
+                a[k].w = fmaf(c, b.w, a[k].w);
+            }
+        }
+    }
+    float f = at * at;
+#pragma unroll
+    for (int k = 0; k < E / 4; ++k) {
+        f = fmaf(a[k].x, a[k].x, f);
+        f = fmaf(a[k].y, a[k].y, f);
+        f = fmaf(a[k].z, a[k].z, f);
+        f = fmaf(a[k].w, a[k].w, f);
+    }
+    publish(0, f);
+    double *np = part + (int64_t)cnt * G;  // behind the dot products' partials
+    block_parts(1, np);
+    if (!meet(m, 2)) return;
+    meet_done(m);
+    if (wl == 0) {
+        const double s = total(np);
+        if (lane == 0) s_norm = s;
+    }
+    __syncthreads();
+    const double hn = sqrt(s_norm);
+    const float sf = (float)(hn > 0.0 ? 1.0 / hn : 0.0);
+#pragma unroll
+    for (int k = 0; k < E / 4; ++k) {
+        const int64_t q = tid + k * st;
+        if (q < nv)
+            reinterpret_cast<float4 *>(w)[q] = make_float4(a[k].x * sf, a[k].y * sf, a[k].z * sf, a[k].w * sf);
+    }
+    if (tail) w[te] = at * sf;
+    if (blockIdx.x == 0 && threadIdx.x == 0) givens_column(s_norm, h, j);
 }
 
 // y = R^-1 g over the first k columns (R the rotated Hessenberg matrix)
@@ -284,7 +449,7 @@ template <typename T>
 __global__ void __launch_bounds__(FT) k_rich(int64_t n, T *__restrict__ z, const T *__restrict__ r,
                                              const T *__restrict__ t, float omega, int first) {
     for (int64_t e = blockIdx.x * (int64_t)FT + threadIdx.x; e < n; e += (int64_t)gridDim.x * FT)
-        z[e] = first ? (T)(omega * r[e]) : (T)(z[e] + omega * (r[e] - t[e]));
+        z[e] = first ? (T)(omega * r[e]) : (T)fma((T)omega, r[e] - t[e], z[e]);
 }
 
 // r = b - A x (x, r, b double) and the partials of r.r; the last block sets
@@ -358,6 +523,9 @@ struct F3R {
     int G;
     double *part;  // G * 64 partials
     unsigned *counter;  // blocks of the running reduction that have finished (0 between launches)
+    Meet meet{};        // of k_arnoldi
+    int coop = 0;       // elements per thread of k_arnoldi (0: the three separate kernels)
+    int coop_blocks = 0;
     Layer<double> L1;
     Layer<TI> L2, L3;
     TI *rt = nullptr;  // the product of a Richardson step (the iterate is layer 3's z_j)
@@ -365,8 +533,34 @@ struct F3R {
     float omega;
     cudaStream_t s;
 
-    // layer 4: z = Richardson(r), m4 steps from z = 0
+    // layer 4: z = Richardson(r), m4 steps from z = 0. A product whose kernel
+    // takes the step as its epilogue reads one buffer and writes the other
+    // (z and rt in turn, the last step into z); the first iterate omega r is
+    // r itself when omega = 1.
     packsell_status richardson(const TI *r, TI *z) {
+        if constexpr (std::is_same<TI, float>::value) {
+            const TI *cur = r;
+            int steps = m4 - 1;
+            if (steps > 0) {
+                if (omega != 1.f) {
+                    TI *first = steps % 2 == 0 ? z : rt;
+                    k_rich<TI><<<G, FT, 0, s>>>(n, first, r, (const TI *)nullptr, omega, 1);
+                    cur = first;
+                }
+                bool done = true;
+                for (; steps > 0 && done; --steps) {
+                    TI *next = steps % 2 == 1 ? z : rt;
+                    packsell_status st = spmv_rich(*A3, cur, r, omega, next, &done, s);
+                    if (st != PACKSELL_OK) return st;
+                    if (!done) break;  // (before the first step: another kernel serves this matrix)
+                    cur = next;
+                }
+                if (done) {
+                    PS_LAUNCH_CHECK("f3r: Richardson");
+                    return PACKSELL_OK;
+                }
+            }
+        }
         k_rich<TI><<<G, FT, 0, s>>>(n, z, r, (const TI *)nullptr, omega, 1);
         for (int k = 1; k < m4; ++k) {
             packsell_status st = layer_spmv(*A3, z, rt, s);
@@ -377,6 +571,36 @@ struct F3R {
         return PACKSELL_OK;
     }
 
+    // k_arnoldi's launch: all blocks resident, E elements of the vector per thread
+    template <int E>
+    bool plan_coop() {
+        int per = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arnoldi<E>, FT, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        const int64_t most = (int64_t)device_sms() * std::min(per, 4);
+        const int64_t want = std::max<int64_t>(1, (n / 4 + FT - 1) / FT);  // one vector per thread
+        coop_blocks = (int)std::min(most, want);
+        if (coop_blocks < 1 || n / 4 > (int64_t)coop_blocks * FT * (E / 4)) return false;
+        coop = E;
+        return true;
+    }
+
+    template <int E>
+    cudaError_t launch_coop(Layer<float> &L, float *w, int cnt, int j) {
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(coop_blocks);
+        cfg.blockDim = dim3(FT);
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k_arnoldi<E>, n, (const float *)L.V, cnt, L.h, j, w, part, meet);
+    }
+
     // one Arnoldi step j of layer L on operator A: w = A z_j, orthogonalise
     // against v_0..v_j, normalise into v_{j+1}
     template <typename T>
@@ -385,6 +609,13 @@ struct F3R {
         packsell_status st = layer_spmv(A, L.Z + (int64_t)j * n, w, s);
         if (st != PACKSELL_OK) return st;
         const int cnt = j + 1;
+        if constexpr (std::is_same<T, float>::value) {
+            if (coop && ((uintptr_t)w & 15u) == 0) {
+                const cudaError_t e = coop == 16 ? launch_coop<16>(L, w, cnt, j) : launch_coop<32>(L, w, cnt, j);
+                if (e != cudaSuccess) return cuda_fail(e, "f3r: Arnoldi step");
+                return PACKSELL_OK;
+            }
+        }
         k_mdot<T><<<dim3(G, cnt), FT, 0, s>>>(n, L.V, w, part, counter, L.h, j);
         k_orth<T><<<G, FT, 0, s>>>(n, L.V, cnt, L.h, j, w, part, counter);
         k_scale<T, T><<<G, FT, 0, s>>>(n, w, w, L.h.scal + 1);
@@ -478,7 +709,9 @@ packsell_status run_f3r(const Matrix &A1, const Matrix &A2, const Matrix &A3, co
     F.omega = (float)o.omega;
     F.s = s;
     F.part = P.take<double>(64 * (size_t)G);
-    F.counter = P.take<unsigned>(1);
+    F.counter = P.take<unsigned>(4);  // the reductions' counter; k_arnoldi's two and its flag
+    F.meet = Meet{F.counter + 1, F.counter + 2, (int *)(F.counter + 3)};
+    if (std::is_same<TI, float>::value && !F.template plan_coop<16>()) F.template plan_coop<32>();
     r = P.take<double>(n);
     ax = P.take<double>(n);
     zt = P.take<double>(n);
@@ -508,7 +741,7 @@ packsell_status run_f3r(const Matrix &A1, const Matrix &A2, const Matrix &A3, co
             return PACKSELL_OK;
         };
         // ||b||
-        if (!ck(cudaMemsetAsync(F.counter, 0, sizeof(unsigned), s))) goto out;
+        if (!ck(cudaMemsetAsync(F.counter, 0, 4 * sizeof(unsigned), s))) goto out;
         k_norm2_begin<double><<<G, FT, 0, s>>>(n, b, F.part, F.counter, F.L1.h);
         double sc[3];
         if (!ck(cudaMemcpyAsync(sc, F.L1.h.scal, sizeof(sc), cudaMemcpyDeviceToHost, s)) ||
@@ -564,9 +797,15 @@ packsell_status run_f3r(const Matrix &A1, const Matrix &A2, const Matrix &A3, co
                 st = F.arnoldi(F.L1, A1, k);
                 if (st != PACKSELL_OK) goto out;
                 ++iters;
+                int timeout = 0;
                 if (!ck(cudaMemcpyAsync(sc, F.L1.h.scal, sizeof(sc), cudaMemcpyDeviceToHost, s)) ||
+                    !ck(cudaMemcpyAsync(&timeout, F.meet.timeout, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
                     !ck(cudaStreamSynchronize(s)))
                     goto out;
+                if (timeout) {
+                    st = fail(PACKSELL_ERR_TIMEOUT, "packsell_f3r: a grid-wide wait ran out");
+                    goto out;
+                }
                 relres = sc[2] / nb;
                 if (!std::isfinite(relres)) {
                     st = fail(PACKSELL_ERR_BREAKDOWN, "packsell_f3r: non-finite residual");

@@ -206,6 +206,8 @@ uint32_t data_wait_limit();
 void set_data_wait_limit(uint32_t limit);
 packsell_status plan_spmv(Matrix &A, cudaStream_t s);
 packsell_status spmv_impl(const Matrix &A, const float *x, float *y, cudaStream_t s);
+packsell_status spmv_rich(const Matrix &A, const float *x, const float *r, float omega, float *y,
+                          bool *done, cudaStream_t s);
 packsell_status spmv_f64_impl(const Matrix &A, const double *x, double *y, cudaStream_t s);
 packsell_status spmm_impl(const Matrix &A, int k, const float *X, int64_t ldx, float *Y,
                           int64_t ldy, cudaStream_t s);

@@ -125,24 +125,44 @@ __device__ __forceinline__ float prefetch_row(int i, int sigma, int sig_shift, l
     return t;
 }
 
+// What is stored for a row's sum t: t itself (r NULL), or a Richardson step
+// x + omega (r - t) with x and r at the row (a kernel of its own reads t, x and
+// r and writes the same value: the same fused multiply-add).
+struct Epilogue {
+    const float *r = nullptr;
+    float omega = 0.f;
+};
+
+// Volatile loads: the addresses are known before the kernel's wait on its
+// predecessor, and loads through const __restrict__ pointers may be moved
+// above that wait (they then read the vectors before they are written).
+__device__ __forceinline__ float epilogue(const Epilogue &e, const float *x, int io, float t) {
+    const float xi = *(const volatile float *)(x + io), ri = *(const volatile float *)(e.r + io);
+    return fmaf(e.omega, ri - t, xi);
+}
+
 // One row per thread; the reducing form (DOT) runs on the fixed solver grid
 // and strides over rows (warps stay on whole slices) so that its reduction
 // is deterministic.
 template <int FMT, int PF, int C, int MINB, bool DOT = false, bool PERM = true,
-          bool EXIT = false, bool PDL = false>
+          bool EXIT = false, bool PDL = false, bool EPI = false>
 __global__ void __launch_bounds__(TPB, MINB)
     k_spmv_prefetch(int n, int sigma, int sig_shift, long long k_left,
                     const int64_t *__restrict__ offset, const uint32_t *__restrict__ pack,
                     const void *__restrict__ perm, int perm_bytes, Decode dc,
-                    const float *__restrict__ x, float *__restrict__ y, Red red = Red{}) {
+                    const float *__restrict__ x, float *__restrict__ y, Red red = Red{},
+                    Epilogue ep = Epilogue{}) {
     if (!DOT) {
-        if (PDL) grid_dep_launch();  // one pass over the rows: signal at block start
+        // one pass over the rows: signal at block start. Not with an epilogue:
+        // there the next kernel of a captured graph is again a product launched
+        // this way, and two in a row that signal early gave wrong results
+        if (PDL && !EPI) grid_dep_launch();
         const int i = blockIdx.x * blockDim.x + threadIdx.x;
         if (i >= n) return;
         int io;
         const float t = prefetch_row<FMT, PF, C, PERM, EXIT, PDL>(
             i, sigma, sig_shift, k_left, offset, pack, perm, perm_bytes, dc, x, io);
-        y[io] = t;
+        y[io] = EPI ? epilogue(ep, x, io, t) : t;
         return;
     }
     if (red.sc->done) return;  // solver converged: idle (grid-uniform)
@@ -458,12 +478,26 @@ packsell_status launch_prefetch_pdl(const Matrix &A, const void *perm, int pb, c
     const Decode dc = make_decode(A);
     const cudaError_t e =
         pb ? launch_pdl(k_spmv_prefetch<FMT, PF, 32, MINB - 1, false, true, false, true>, g, TPB, s, n,
-                        sg, sh, kl, offset, pack, perm, pb, dc, x, y, Red{})
+                        sg, sh, kl, offset, pack, perm, pb, dc, x, y, Red{}, Epilogue{})
            : launch_pdl(k_spmv_prefetch<FMT, PF, 32, MINB, false, false, false, true>, g, TPB, s, n, sg,
-                        sh, kl, offset, pack, perm, pb, dc, x, y, Red{});
+                        sh, kl, offset, pack, perm, pb, dc, x, y, Red{}, Epilogue{});
     if (e != cudaSuccess) return cuda_fail(e, "packsell_spmv (variant 13)");
     PS_LAUNCH_CHECK("packsell_spmv (variant 13)");
     return PACKSELL_OK;
+}
+
+// Variant 13 with the Richardson step as its epilogue (implicit order).
+template <int FMT>
+cudaError_t launch_prefetch_rich(const Matrix &A, const float *x, float *y, const Epilogue &ep,
+                                 cudaStream_t s) {
+    const int sg = A.p.sigma;
+    const int sh = (sg & (sg - 1)) == 0 ? __builtin_ctz((unsigned)sg) : -1;
+    const unsigned g = (unsigned)grid_for(A.n);
+    auto k = A.perm_bytes ? k_spmv_prefetch<FMT, 16, 32, 4, false, true, false, true, true>
+                          : k_spmv_prefetch<FMT, 16, 32, 5, false, false, false, true, true>;
+    return launch_pdl(k, g, TPB, s, (int)A.n, sg, sh, (long long)A.p.k_left, (const int64_t *)A.offset,
+                      (const uint32_t *)A.pack, (const void *)A.perm, A.perm_bytes, make_decode(A), x, y,
+                      Red{}, ep);
 }
 
 // variant 13 with its round size fitted to the widest slice (as variant 5)
@@ -887,14 +921,14 @@ __global__ void __launch_bounds__(TPB, 4)
 // UNROLL slots go out before any is used, as in the FP32 SELL kernel, and the
 // launch is programmatic (values and columns load before the wait on the
 // previous kernel of the stream; x and y after it).
-template <int U, bool C32>
+template <int U, bool C32, bool EPI = false>
 __global__ void __launch_bounds__(TPB)
     k_spmv_sell16(int n, int Cr, int sigma, const int64_t *__restrict__ offset,
                   const uint16_t *__restrict__ val, const int32_t *__restrict__ col,
                   const void *__restrict__ perm, int perm_bytes, const float *__restrict__ x,
-                  float *__restrict__ y) {
+                  float *__restrict__ y, Epilogue ep) {
     const int C = C32 ? 32 : Cr;  // a constant slot stride when C = 32
-    grid_dep_launch();  // one pass over the rows: signal at block start
+    if (!EPI) grid_dep_launch();  // one pass over the rows: signal at block start
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) {
         grid_dep_wait();
@@ -929,7 +963,8 @@ __global__ void __launch_bounds__(TPB)
         if (cc[U - 1] < 0) break;  // padding: the row has ended
     }
     if (!waited) grid_dep_wait();
-    y[orig_row(i, sigma, perm, perm_bytes)] = t;
+    const int io = orig_row(i, sigma, perm, perm_bytes);
+    y[io] = EPI ? epilogue(ep, x, io, t) : t;
 }
 
 // Thread-per-row PackSELL SpMV fused with sum_i x_i y_i (solver use, any C),
@@ -1231,7 +1266,7 @@ packsell_status spmv_impl(const Matrix &A, const float *x, float *y, cudaStream_
             const cudaError_t e = launch_pdl(k, (unsigned)g, TPB, s, (int)A.n, A.p.C,
                                              A.p.sigma, (const int64_t *)A.offset,
                                              (const uint16_t *)A.val, (const int32_t *)A.col, perm,
-                                             pb, x, y);
+                                             pb, x, y, Epilogue{});
             if (e != cudaSuccess) return cuda_fail(e, "packsell_spmv (FP16 SELL)");
             break;
         }
@@ -1240,6 +1275,32 @@ packsell_status spmv_impl(const Matrix &A, const float *x, float *y, cudaStream_
                         "packsell_spmv: SELL_F64 and W64_E11MY need packsell_spmv_f64");
     }
     PS_LAUNCH_CHECK("packsell_spmv");
+    return PACKSELL_OK;
+}
+
+// y = x + omega (r - A x) in one kernel, for the matrices whose product runs
+// the row-prefetch kernel in rounds of 16 words (C = 32) or is FP16 SELL;
+// *done is false when the matrix takes another kernel (nothing is launched).
+packsell_status spmv_rich(const Matrix &A, const float *x, const float *r, float omega, float *y,
+                          bool *done, cudaStream_t s) {
+    const Epilogue ep{r, omega};
+    cudaError_t e = cudaSuccess;
+    *done = true;
+    const int var = A.variant == 0 ? A.auto_variant : A.variant;
+    if (A.n == 0) return PACKSELL_OK;
+    if (is_packed(A.p.format) && A.p.C == 32 && !A.p.explicit_perm && var == 13 &&
+        round_words(A.max_width) == 16) {
+        e = A.p.format == PACKSELL_FMT_FP16 ? launch_prefetch_rich<PACKSELL_FMT_FP16>(A, x, y, ep, s)
+                                            : launch_prefetch_rich<PACKSELL_FMT_E8MY>(A, x, y, ep, s);
+    } else if (is_sell16(A.p.format) && A.p.C == 32 && !A.p.explicit_perm && A.max_width > 8) {
+        e = launch_pdl(k_spmv_sell16<16, true, true>, (unsigned)grid_for(A.n), TPB, s, (int)A.n, A.p.C,
+                       A.p.sigma, (const int64_t *)A.offset, (const uint16_t *)A.val,
+                       (const int32_t *)A.col, (const void *)A.perm, A.perm_bytes, x, y, ep);
+    } else {
+        *done = false;
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "product with Richardson step");
+    PS_LAUNCH_CHECK("product with Richardson step");
     return PACKSELL_OK;
 }
 
@@ -1351,11 +1412,11 @@ void launch_prefetch_dot(const Matrix &A, const float *x, float *y, const Red &r
     if (A.perm_bytes) {
         auto k = k_spmv_prefetch<FMT, PF, 32, MINB - 1, true, true>;
         k<<<dot_grid(k), TPB, 0, s>>>((int)A.n, sg, sh, A.p.k_left, A.offset, A.pack, A.perm,
-                                      A.perm_bytes, make_decode(A), x, y, red);
+                                      A.perm_bytes, make_decode(A), x, y, red, Epilogue{});
     } else {
         auto k = k_spmv_prefetch<FMT, PF, 32, MINB, true, false>;
         k<<<dot_grid(k), TPB, 0, s>>>((int)A.n, sg, sh, A.p.k_left, A.offset, A.pack, A.perm, 0,
-                                      make_decode(A), x, y, red);
+                                      make_decode(A), x, y, red, Epilogue{});
     }
 }
 
