@@ -37,6 +37,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "meet.cuh"
 
 namespace packsell {
 
@@ -50,16 +51,27 @@ inline int fgrid(int64_t n) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)device_sms() * 4, (n + FT - 1) / FT));
 }
 
-// block-wide sum of a double (fixed tree), result in thread 0
-__device__ __forceinline__ double block_sum(double v, double *sh) {
+// sum of the block's FT values in shared memory by one warp (every lane has
+// it): 13 FP64 additions where a shuffle tree in all eight warps takes 40 (an
+// FP64 warp instruction takes about 16 cycles of an SM)
+template <typename T>
+__device__ __forceinline__ double warp_total(const T *v, int lane) {
+    double x[FT / 32], t = 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
+    for (int q = 0; q < FT / 32; ++q) x[q] = (double)v[32 * q + lane];
+#pragma unroll
+    for (int q = 0; q < FT / 32; ++q) t += x[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+// block-wide sum of a double (fixed order), result in thread 0; sh: FT values
+__device__ __forceinline__ double block_sum(double v, double *sh) {
+    sh[threadIdx.x] = v;
     __syncthreads();
     double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[k];
+    if (threadIdx.x < 32) t = warp_total(sh, threadIdx.x);
     __syncthreads();
     return t;
 }
@@ -93,7 +105,13 @@ __device__ __forceinline__ bool last_block(unsigned *counter) {
 // sum of the G partials at p, in block order (the whole block; thread 0 has it)
 __device__ __forceinline__ double partial_sum(const double *p, int G, double *sh) {
     double s = 0.0;
-    for (int b = threadIdx.x; b < G; b += FT) s += ((const volatile double *)p)[b];
+    for (int b0 = threadIdx.x; b0 < G; b0 += 4 * FT) {  // the loads together, then the additions
+        double v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = b0 + q * FT < G ? ((const volatile double *)p)[b0 + q * FT] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s += v[q];
+    }
     return block_sum(s, sh);
 }
 
@@ -115,7 +133,7 @@ template <typename T>
 __global__ void __launch_bounds__(FT) k_norm2_begin(int64_t n, const T *__restrict__ v,
                                                     double *__restrict__ part, unsigned *counter,
                                                     Hess h) {
-    __shared__ double sh[FT / 32];
+    __shared__ double sh[FT];
     double s = 0.0;
     if constexpr (std::is_same<T, float>::value) {  // an FP32 layer: FP32 thread partials
         float sf = 0.f;
@@ -139,7 +157,7 @@ template <typename T>
 __global__ void __launch_bounds__(FT) k_mdot(int64_t n, const T *__restrict__ V,
                                              const T *__restrict__ w, double *__restrict__ part,
                                              unsigned *counter, Hess h, int j) {
-    __shared__ double sh[FT / 32];
+    __shared__ double sh[FT];
     const T *__restrict__ v = V + (int64_t)blockIdx.y * n;
     double s = 0.0;
     if constexpr (std::is_same<T, float>::value) {
@@ -212,7 +230,7 @@ template <typename T>
 __global__ void __launch_bounds__(FT) k_orth(int64_t n, const T *__restrict__ V, int cnt, Hess h, int j,
                                              T *__restrict__ w, double *__restrict__ part,
                                              unsigned *counter) {
-    __shared__ double sh[FT / 32];
+    __shared__ double sh[FT];
     __shared__ double hc[64];
     __shared__ float hf[64];
     for (int i = threadIdx.x; i < cnt; i += FT) {
@@ -253,44 +271,12 @@ __global__ void __launch_bounds__(FT) k_orth(int64_t n, const T *__restrict__ V,
 // registers through the dot products, the update and the scaling, and the
 // blocks (all resident: a cooperative launch) meet twice. Every block adds
 // all partials itself, in block order, so all have the same sums.
-struct Meet {
-    unsigned *arrived, *left;  // 0 between launches
-    int *timeout;              // set when a wait ran out: later launches return at once
-};
-
-constexpr unsigned kMeetPolls = 1u << 22;
-
-// Wait (bounded) until all blocks have arrived `round` times; false when the wait ran out.
-__device__ __forceinline__ bool meet(const Meet &m, unsigned round) {
-    __shared__ bool ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(m.arrived, 1u);
-        const unsigned all = gridDim.x * round;
-        unsigned polls = 0;
-        while (*(volatile unsigned *)m.arrived < all && ++polls < kMeetPolls) __nanosleep(32);
-        ok = polls < kMeetPolls;
-        if (!ok) *m.timeout = 1;
-        __threadfence();
-    }
-    __syncthreads();
-    return ok;
-}
-
-// The last block to call this after the last meet() puts the counters back.
-__device__ __forceinline__ void meet_done(const Meet &m) {
-    if (threadIdx.x == 0 && atomicAdd(m.left, 1u) == gridDim.x - 1u) {
-        *m.arrived = 0u;
-        *m.left = 0u;
-    }
-}
-
 template <int E>
 __global__ void __launch_bounds__(FT, 4)
     k_arnoldi(int64_t n, const float *__restrict__ V, int cnt, Hess h, int j, float *__restrict__ w,
               double *__restrict__ part, Meet m) {
-    __shared__ double sh[64][FT / 32];
+    constexpr int PB = 8;  // quantities reduced together, one per warp
+    __shared__ float sh[PB][FT];
     __shared__ float hf[64];
     __shared__ double s_norm;
     if (*(volatile int *)m.timeout) return;
@@ -306,29 +292,31 @@ __global__ void __launch_bounds__(FT, 4)
     const int64_t te = nv * 4 + tid;
     const bool tail = te < n;
     float at = tail ? w[te] : 0.f;
-    // the lanes' sums of one quantity into sh[i][warp]
-    auto publish = [&](int i, float f) {
-        double d = (double)f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (lane == 0) sh[i][wl] = d;
-    };
     // the grid's sum of one quantity, every lane of the warp (partials in block order)
     auto total = [&](const double *p) {
         double s = 0.0;
-        for (int b = lane; b < G; b += 32) s += ((const volatile double *)p)[b];
+        for (int b0 = 0; b0 < G; b0 += 8 * 32) {  // eight loads in flight, added in order
+            double v[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int b = b0 + 32 * q + lane;
+                v[q] = b < G ? ((const volatile double *)p)[b] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) s += v[q];
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         return s;
     };
-    auto block_parts = [&](int count, double *out) {  // sh -> one partial per block and quantity
+    // the block's sums of the quantities [i0, i0 + count) in sh, one partial each
+    auto block_parts = [&](int i0, int count, double *out) {
         __syncthreads();
-        for (int i = threadIdx.x; i < count; i += FT) {
-            double s = 0.0;
-#pragma unroll
-            for (int q = 0; q < FT / 32; ++q) s += sh[i][q];
-            out[(int64_t)i * G + blockIdx.x] = s;
+        if (wl < count) {
+            const double s = warp_total(sh[wl], lane);
+            if (lane == 0) out[(int64_t)(i0 + wl) * G + blockIdx.x] = s;
         }
+        __syncthreads();
     };
     for (int i = 0; i < cnt; ++i) {
         const float *__restrict__ v = V + (int64_t)i * n;
@@ -346,9 +334,9 @@ __global__ void __launch_bounds__(FT, 4)
                 f = fmaf(a[k].w, b.w, f);
             }
         }
-        publish(i, f);
+        sh[i % PB][threadIdx.x] = f;
+        if (i % PB == PB - 1 || i + 1 == cnt) block_parts(i / PB * PB, i % PB + 1, part);
     }
-    block_parts(cnt, part);
     if (!meet(m, 1)) return;
     for (int i = wl; i < cnt; i += FT / 32) {
         const double s = total(part + (int64_t)i * G);
@@ -384,9 +372,9 @@ __global__ void __launch_bounds__(FT, 4)
         f = fmaf(a[k].z, a[k].z, f);
         f = fmaf(a[k].w, a[k].w, f);
     }
-    publish(0, f);
+    sh[0][threadIdx.x] = f;
     double *np = part + (int64_t)cnt * G;  // behind the dot products' partials
-    block_parts(1, np);
+    block_parts(0, 1, np);
     if (!meet(m, 2)) return;
     meet_done(m);
     if (wl == 0) {
@@ -457,7 +445,7 @@ __global__ void __launch_bounds__(FT) k_rich(int64_t n, T *__restrict__ z, const
 __global__ void __launch_bounds__(FT) k_resid(int64_t n, const double *__restrict__ b,
                                               const double *__restrict__ ax, double *__restrict__ r,
                                               double *__restrict__ part, unsigned *counter, Hess h) {
-    __shared__ double sh[FT / 32];
+    __shared__ double sh[FT];
     double s = 0.0;
     for (int64_t e = blockIdx.x * (int64_t)FT + threadIdx.x; e < n; e += (int64_t)gridDim.x * FT) {
         const double v = b[e] - ax[e];
@@ -588,17 +576,9 @@ struct F3R {
     }
 
     template <int E>
-    cudaError_t launch_coop(Layer<float> &L, float *w, int cnt, int j) {
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(coop_blocks);
-        cfg.blockDim = dim3(FT);
-        cfg.stream = s;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, k_arnoldi<E>, n, (const float *)L.V, cnt, L.h, j, w, part, meet);
+    cudaError_t launch_step(Layer<float> &L, float *w, int cnt, int j) {
+        return launch_coop(k_arnoldi<E>, (unsigned)coop_blocks, FT, 0, s, n, (const float *)L.V, cnt, L.h,
+                           j, w, part, meet);
     }
 
     // one Arnoldi step j of layer L on operator A: w = A z_j, orthogonalise
@@ -611,7 +591,7 @@ struct F3R {
         const int cnt = j + 1;
         if constexpr (std::is_same<T, float>::value) {
             if (coop && ((uintptr_t)w & 15u) == 0) {
-                const cudaError_t e = coop == 16 ? launch_coop<16>(L, w, cnt, j) : launch_coop<32>(L, w, cnt, j);
+                const cudaError_t e = coop == 16 ? launch_step<16>(L, w, cnt, j) : launch_step<32>(L, w, cnt, j);
                 if (e != cudaSuccess) return cuda_fail(e, "f3r: Arnoldi step");
                 return PACKSELL_OK;
             }

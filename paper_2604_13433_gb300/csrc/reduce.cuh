@@ -130,34 +130,50 @@ __device__ __forceinline__ void finish(const Red &r, double s1, double s2) {
     }
 }
 
-// Sum (v1, v2) over the block (blockDim.x a multiple of 32, at most 1024).
-__device__ __forceinline__ void block_sum2(double &v1, double &v2) {
-    __shared__ double s1[32], s2[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-        v1 += __shfl_down_sync(0xffffffffu, v1, o);
-        v2 += __shfl_down_sync(0xffffffffu, v2, o);
-    }
+// Sum (v1, v2) over a block of RED_TPB threads, in thread 0; v2 only with
+// `two`. GB300's FP64 pipe takes about 16 cycles per warp instruction, so a
+// tree of shuffles in every warp (40 additions per value and block of eight
+// warps) cost 2.5 us of FP64 issue per SM and reducing kernel, with four
+// blocks per SM. Here one warp per value adds the threads' values from shared
+// memory: 13 additions.
+constexpr int RED_TPB = 256;
+
+__device__ __forceinline__ void block_sum2(double &v1, double &v2, bool two) {
+    __shared__ double s[2][RED_TPB];
+    __shared__ double s2;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();  // the arrays may still be read by a previous call
-    if (lane == 0) {
-        s1[wid] = v1;
-        s2[wid] = v2;
-    }
+    s[0][threadIdx.x] = v1;
+    if (two) s[1][threadIdx.x] = v2;
     __syncthreads();
-    if (wid == 0) {
-        v1 = lane < nw ? s1[lane] : 0.0;
-        v2 = lane < nw ? s2[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            v1 += __shfl_down_sync(0xffffffffu, v1, o);
-            v2 += __shfl_down_sync(0xffffffffu, v2, o);
-        }
+    if (wid == 0 || (two && wid == 1)) {
+        double v[RED_TPB / 32], t = 0.0;
+#pragma unroll
+        for (int q = 0; q < RED_TPB / 32; ++q) v[q] = s[wid][32 * q + lane];
+#pragma unroll
+        for (int q = 0; q < RED_TPB / 32; ++q) t += v[q];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (wid == 0) v1 = t;
+        else if (lane == 0) s2 = t;
     }
+    if (two) {
+        __syncthreads();
+        v2 = s2;
+    } else {
+        v2 = 0.0;
+    }
+}
+
+// finish steps that use their second sum
+__device__ __forceinline__ bool uses_second(int fin) {
+    return fin == FIN_RZ_BETA_RR || fin == FIN_OUTER_ALPHA || fin == FIN_BB_RR;
 }
 
 // Every thread of every block calls this once with its contributions.
 __device__ __forceinline__ void reduce_publish(const Red &r, double v1, double v2) {
     __shared__ bool last;
-    block_sum2(v1, v2);
+    const bool two = uses_second(r.fin);
+    block_sum2(v1, v2, two);
     if (threadIdx.x == 0) {
         r.partials[2 * blockIdx.x] = v1;
         r.partials[2 * blockIdx.x + 1] = v2;
@@ -167,12 +183,25 @@ __device__ __forceinline__ void reduce_publish(const Red &r, double v1, double v
     __syncthreads();
     if (!last) return;
     __threadfence();
+    // the partials of a thread load together (added one by one they cost the
+    // kernel's tail a trip to the L2 each: 6 us with 912 blocks and two sums)
+    constexpr int U = 6;
     double a = 0.0, b = 0.0;
-    for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
-        a += ((volatile double *)r.partials)[2 * q];
-        b += ((volatile double *)r.partials)[2 * q + 1];
+    for (unsigned q0 = threadIdx.x; q0 < gridDim.x; q0 += U * blockDim.x) {
+        double va[U], vb[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned q = q0 + u * blockDim.x;
+            va[u] = q < gridDim.x ? ((volatile double *)r.partials)[2 * q] : 0.0;
+            vb[u] = two && q < gridDim.x ? ((volatile double *)r.partials)[2 * q + 1] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            a += va[u];
+            if (two) b += vb[u];
+        }
     }
-    block_sum2(a, b);
+    block_sum2(a, b, two);
     if (threadIdx.x == 0) {
         finish(r, a, b);
         *r.counter = 0u;
