@@ -149,6 +149,81 @@ __global__ void __launch_bounds__(TPB)
     }
 }
 
+// Lane groups with 32-byte X and Y rows: a lane owns eight neighbouring columns
+// and fetches them with one 256-bit load (sm_100 and later), G lanes a row of
+// 8 G columns. What bounded the kernel above at k = 16 on the 27-point matrix
+// was the L1: a warp's 16-byte loads of every other quarter row used 32 bytes
+// of each line they touched, 8.6 line accesses per load and two loads per word
+// (L1 95 % busy). Here one load takes the same 16 rows whole. At k = 64 it was
+// instruction issue (47 instructions per word and lane group: 64-bit address
+// arithmetic, column predicates, eight multiply-adds); here the row address is
+// one 32 x 32-bit multiply-add, a lane's columns are all in or all out, and two
+// columns share a multiply-add (fma.rn.f32x2, each half rounds as fmaf does).
+// Each column keeps its stored-order chain. Measured on the 27-point 128^3
+// matrix, before and after: k = 8 127 / 95 us, 16 228 / 171, 32 438 / 331,
+// 64 698 / 629. What is left is latency (long-scoreboard stalls 14 cycles per
+// issue at 68 % of the warps): a second word's load in flight needs registers
+// that cost a block per SM (178 us at k = 16), four of them spill.
+struct Cols8 {
+    unsigned long long v[4];
+};
+
+__device__ __forceinline__ Cols8 load8(const void *p) {
+    Cols8 r;
+    asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];"
+        : "=l"(r.v[0]), "=l"(r.v[1]), "=l"(r.v[2]), "=l"(r.v[3])
+        : "l"(p));
+    return r;
+}
+
+__device__ __forceinline__ void store8(void *p, const Cols8 &r) {
+    asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(r.v[0]), "l"(r.v[1]), "l"(r.v[2]),
+                 "l"(r.v[3])
+                 : "memory");
+}
+
+__device__ __forceinline__ void fma8(Cols8 &a, float v, const Cols8 &x) {
+    unsigned long long vv;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(vv) : "f"(v));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a.v[q]) : "l"(vv), "l"(x.v[q]));
+}
+
+template <int FMT, int G>
+__global__ void __launch_bounds__(TPB, 6)
+    k_spmm_wide(int n, int sigma, long long k_left, const int64_t *__restrict__ offset,
+                const uint32_t *__restrict__ pack, const void *__restrict__ perm, int perm_bytes,
+                Decode dc, int k, const float *__restrict__ X, uint32_t xstride, float *__restrict__ Y,
+                int64_t ldy) {
+    const int i = (int)(((int64_t)blockIdx.x * TPB + threadIdx.x) / G), sub = threadIdx.x % G;
+    if (i >= n) return;
+    const int64_t s = offset[i >> 5];
+    const int w = (int)((offset[(i >> 5) + 1] - s) >> 5);
+    const uint32_t *__restrict__ pp = pack + s + (i & 31);
+    const int c0 = left_offset(i, sigma, k_left);
+    const int io = orig_row(i, sigma, perm, perm_bytes);
+    for (int q0 = 8 * sub; q0 < k; q0 += 8 * G) {
+        const char *__restrict__ xq = reinterpret_cast<const char *>(X + q0);
+        Cols8 acc = {};
+        uint32_t c = (uint32_t)c0;
+        for (int j0 = 0; j0 < w; j0 += SPF) {
+            const int wr = w - j0;
+            uint32_t wd[SPF];
+#pragma unroll
+            for (int u = 0; u < SPF; ++u) wd[u] = (u < wr) ? ldg_stream(pp + (j0 + u) * 32) : 0u;
+#pragma unroll
+            for (int u = 0; u < SPF; ++u) {
+                const bool f = (wd[u] & 1u) != 0u;
+                c += (wd[u] >> 1) & (f ? dc.dmask : 0x7fffffffu);
+                if (f && PS_IN_RANGE(c, dc.xlen))
+                    fma8(acc, word_value<FMT>(wd[u], dc), load8(xq + (uint64_t)c * xstride));
+            }
+            if (wd[SPF - 1] == 0u) break;  // the row has ended
+        }
+        store8(Y + (int64_t)io * ldy + q0, acc);
+    }
+}
+
 // The same lane-group SpMM for FP32 SELL: every stored slot multiplies
 // (padding holds value 0), as in the SELL SpMV.
 template <int G, int KV, bool VEC>
@@ -217,6 +292,23 @@ void launch_spmm_v(bool vec, const Matrix &A, const void *perm, int pb, int k, c
     else launch_spmm<G, KV, false>(A, perm, pb, k, X, ldx, Y, ldy, s);
 }
 
+template <int FMT, int G>
+void launch_wide(const Matrix &A, const void *perm, int pb, int k, const float *X, int64_t ldx, float *Y,
+                 int64_t ldy, cudaStream_t s) {
+    const unsigned g = (unsigned)((A.n * G + TPB - 1) / TPB);
+    k_spmm_wide<FMT, G><<<g, TPB, 0, s>>>((int)A.n, A.p.sigma, A.p.k_left, A.offset, A.pack, perm, pb, make_decode(A), k,
+                           X, (uint32_t)(ldx * sizeof(float)), Y, ldy);
+}
+
+template <int FMT>
+void launch_wide_k(const Matrix &A, const void *perm, int pb, int k, const float *X, int64_t ldx, float *Y,
+                   int64_t ldy, cudaStream_t s) {
+    if (k <= 8) launch_wide<FMT, 1>(A, perm, pb, k, X, ldx, Y, ldy, s);
+    else if (k <= 16) launch_wide<FMT, 2>(A, perm, pb, k, X, ldx, Y, ldy, s);
+    else if (k <= 32) launch_wide<FMT, 4>(A, perm, pb, k, X, ldx, Y, ldy, s);
+    else launch_wide<FMT, 8>(A, perm, pb, k, X, ldx, Y, ldy, s);
+}
+
 packsell_status spmm_impl(const Matrix &A, int k, const float *X, int64_t ldx, float *Y,
                           int64_t ldy, cudaStream_t s) {
     if (k < 1 || ldx < k || ldy < k)
@@ -235,6 +327,16 @@ packsell_status spmm_impl(const Matrix &A, int k, const float *X, int64_t ldx, f
                                                 (const MultiItem *)A.multi_items, A.multi_nitems, k,
                                                 vec, s);
         return st;
+    }
+    // 32-byte rows and slices of at most 48 words: eight columns per lane
+    if (A.p.C == 32 && is_packed(A.p.format) && A.max_width <= 48 && k % 8 == 0 && ldx % 8 == 0 &&
+        ldy % 8 == 0 && ldx < (1ll << 30) && ((uintptr_t)X & 31) == 0 && ((uintptr_t)Y & 31) == 0) {
+        if (A.p.format == PACKSELL_FMT_FP16)
+            launch_wide_k<PACKSELL_FMT_FP16>(A, perm, pb, k, X, ldx, Y, ldy, s);
+        else
+            launch_wide_k<PACKSELL_FMT_E8MY>(A, perm, pb, k, X, ldx, Y, ldy, s);
+        PS_LAUNCH_CHECK("packsell_spmm");
+        return PACKSELL_OK;
     }
     // lanes per row and column groups per lane: one pass for k <= 128
     if (k <= 4) launch_spmm_v<1, 1>(vec, A, perm, pb, k, X, ldx, Y, ldy, s);
