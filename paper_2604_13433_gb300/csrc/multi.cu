@@ -431,10 +431,15 @@ __device__ __forceinline__ void rows_store(const SplitMat &M, float *__restrict_
     }
 }
 
-// words of a round per lane group: four gathers in flight per lane
+// words of a round per lane group. With two column groups per lane eight
+// 16-byte gathers are in flight and the kernel runs two blocks per SM: 530 ->
+// 497 us at k = 64 on the power-law matrix of 1M rows, 127 -> 108 us on 60,000
+// rows (four gathers and three blocks before; a 4,096-word row is one warp's
+// work, 512 words' gathers one after another). With one group, four gathers
+// and three blocks (k = 32: 401 us; eight and two 403, eight and three 481).
 template <int NQ>
 constexpr int rows_round() {
-    return NQ >= 4 ? 1 : 4 / NQ;
+    return 4;
 }
 
 // A tile: the words are split into RPI runs of about nwd / RPI words, each
@@ -626,7 +631,7 @@ __device__ __forceinline__ void rows_long(const SplitMat &M, int row, long long 
 // Persistent grid over the same items as k_split_multi, the next item's words
 // and row offsets loading while the current one is processed.
 template <int KG, int NQ, bool SINGLE>
-__global__ void __launch_bounds__(MW * 32, SINGLE ? 3 : 2)
+__global__ void __launch_bounds__(MW * 32, SINGLE && NQ == 1 ? 3 : 2)
     k_split_rows(SplitMat M0, const SplitMat *__restrict__ mats, const MultiItem *__restrict__ items,
                  int nitems) {
     __shared__ __align__(16) uint32_t s_lft[MW][MT];
