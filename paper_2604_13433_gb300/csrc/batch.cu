@@ -50,7 +50,7 @@ struct Batch {
     bool vec = false;  // every X and Y allows 16-byte accesses
     SplitMat *d_smats = nullptr;
     MultiItem *d_mitems = nullptr;
-    int n_mitems = 0;
+    int n_mitems = 0, n_mlong = 0;  // n_mlong: single long rows, the first items
     bool split1 = false;  // the items are variant 14's (one right-hand side)
     bool sorted = false;  // a CSR-order matrix has sigma > 1
 };
@@ -152,6 +152,7 @@ static packsell_status upload_split(Batch *B, const std::vector<SplitMat> &smats
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "packsell_batch_create: plan copy");
     B->n_mitems = (int)mitems.size();
+    B->n_mlong = (int)std::count_if(mitems.begin(), mitems.end(), [](const MultiItem &a) { return a.meta < 0; });
     return PACKSELL_OK;
 }
 
@@ -225,11 +226,7 @@ packsell_status batch_create(int count, const Matrix *const *A, const float *con
         }
         if (m->p.C == 1) {
             B->sorted = B->sorted || m->p.sigma > 1;
-            const packsell_status st = split_items_append(offs.data(), m->n, i, mitems);
-            if (st != PACKSELL_OK) {
-                batch_free(B);
-                return st;
-            }
+            split_items_append(offs.data(), m->n, i, mitems);
             continue;
         }
         int k0 = 0;
@@ -321,11 +318,7 @@ packsell_status batch_create_mm(int count, const Matrix *const *A, int k, const 
         if (A[i]->n == 0) continue;
         const std::vector<int64_t> &o = offs_all[j++];
         if (split1) {
-            const packsell_status st = split_items_append(o.data(), A[i]->n, i, mitems);
-            if (st != PACKSELL_OK) {
-                batch_free(B);
-                return st;
-            }
+            split_items_append(o.data(), A[i]->n, i, mitems);
         } else {
             multi_items_append(o.data(), A[i]->n, i, mitems);
         }
@@ -353,13 +346,13 @@ packsell_status batch_spmv(const Batch &B, cudaStream_t s) {
         k_spmv_batched<<<B.blocks, BTPB, 0, s>>>(B.d_mats, B.d_items, B.nitems);
         PS_LAUNCH_CHECK("packsell_batch_spmv");
     }
-    return launch_split_batch(B.d_smats, B.d_mitems, B.n_mitems, B.sorted, s);
+    return launch_split_batch(B.d_smats, B.d_mitems, B.n_mitems, B.n_mlong, B.sorted, s);
 }
 
 packsell_status batch_spmm(const Batch &B, cudaStream_t s) {
     if (B.d_mats)
         return fail(PACKSELL_ERR_INVALID_ARG, "packsell_batch_spmm: the plan is a batched SpMV plan");
-    if (B.split1) return launch_split_batch(B.d_smats, B.d_mitems, B.n_mitems, B.sorted, s);
+    if (B.split1) return launch_split_batch(B.d_smats, B.d_mitems, B.n_mitems, B.n_mlong, B.sorted, s);
     return launch_multi(SplitMat{}, B.d_smats, B.d_mitems, B.n_mitems, B.k, B.vec, s);
 }
 

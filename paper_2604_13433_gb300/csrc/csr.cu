@@ -34,6 +34,7 @@ namespace {
 constexpr int CT = 256;  // words per tile (and per chunk of a long row)
 constexpr int CR = 64;   // rows per tile at most
 constexpr int CL = 256;  // rows of more words take the warp-cooperative path
+static_assert(CL == CT, "a row is a tile or long");
 constexpr int CW = 8;    // warps per block
 constexpr int CPF = 8;   // words of a row gathered at once (most rows are short)
 
@@ -216,45 +217,7 @@ void csr_plan_free(Matrix &A, const Release &rel) {
 // most CL words are grouped greedily while they hold at most CT words and CR
 // rows; a row of more than CL words is an item of its own. Built on the host
 // from the row offsets.
-packsell_status plan_csr(Matrix &A, cudaStream_t s) {
-    if (!is_packed(A.p.format) || A.p.C != 1 || A.n == 0) return PACKSELL_OK;
-    std::vector<int64_t> off((size_t)A.n + 1);
-    PS_CUDA(cudaMemcpyAsync(off.data(), A.offset, sizeof(int64_t) * (A.n + 1),
-                            cudaMemcpyDeviceToHost, s));
-    PS_CUDA(cudaStreamSynchronize(s));
-    std::vector<int2> items;
-    items.reserve((size_t)(A.n_words / CT + A.n / CR + 16));
-    int r0 = 0;
-    for (int r = 0; r < (int)A.n; ++r) {
-        const int64_t w = off[r + 1] - off[r];
-        if (w > CL) {  // a long row: close the tile before it, then the row alone
-            if (r > r0) items.push_back(make_int2(r0, r));
-            items.push_back(make_int2(r, r + 1));
-            r0 = r + 1;
-            continue;
-        }
-        if (off[r + 1] - off[r0] > CT || r + 1 - r0 > CR) {
-            items.push_back(make_int2(r0, r));
-            r0 = r;
-        }
-    }
-    if ((int)A.n > r0) items.push_back(make_int2(r0, (int)A.n));
-    // long rows first, longest first: they set the kernel's critical path,
-    // and taken early from the queue they overlap the many short tiles
-    auto is_long = [&](const int2 &a) { return a.y - a.x == 1 && off[a.y] - off[a.x] > CL; };
-    std::stable_partition(items.begin(), items.end(), is_long);
-    const size_t nlong = (size_t)std::count_if(items.begin(), items.end(), is_long);
-    std::stable_sort(items.begin(), items.begin() + nlong, [&](const int2 &a, const int2 &b) {
-        return off[a.y] - off[a.x] > off[b.y] - off[b.x];
-    });
-    if (items.size() >= (size_t)INT32_MAX) return fail(PACKSELL_ERR_RANGE, "plan_csr: too many items");
-    PS_CUDA(pool_get(&A.csr_items, sizeof(int2) * items.size(), s));
-    PS_CUDA(cudaMemcpyAsync(A.csr_items, items.data(), sizeof(int2) * items.size(),
-                            cudaMemcpyHostToDevice, s));
-    PS_CUDA(cudaStreamSynchronize(s));
-    A.csr_nitems = (int)items.size();
-    return PACKSELL_OK;
-}
+CutRule csr_rule() { return CutRule{CUT_CSR, CL, CR}; }
 
 packsell_status launch_csr(const Matrix &A, const void *perm, int pb, const float *x, float *y,
                            cudaStream_t s) {

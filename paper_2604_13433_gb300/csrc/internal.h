@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -143,7 +144,6 @@ packsell_status spmv_w16_impl(const Matrix &A, const float *x, float *y, cudaStr
 packsell_status spmv_x16_impl(const Matrix &A, const uint16_t *x, uint16_t *y, cudaStream_t s);
 
 // csr.cu
-packsell_status plan_csr(Matrix &A, cudaStream_t s);
 void csr_plan_free(Matrix &A, const Release &rel);
 packsell_status launch_csr(const Matrix &A, const void *perm, int pb, const float *x, float *y,
                            cudaStream_t s);
@@ -169,20 +169,53 @@ struct __align__(16) MultiItem {  // a tile (meta = rows << 16 | words) or a lon
     int mat;
     int pad0, pad1, pad2;
 };
+// Work item of variant 14: a tile of rows [r0, r0 + nrows) holding nwd words
+// from word `base` (meta = nrows << 16 | nwd), or one long row of nwd words
+// (meta = -nwd). One 16-byte load gives a warp everything it needs to start.
+struct __align__(16) SplitItem {
+    long long base;
+    int r0;
+    int meta;
+};
+
+// items.cu: how the rows of a CSR-order (C = 1) matrix are cut into items
+enum CutKind { CUT_CSR, CUT_SPLIT, CUT_MULTI };
+struct CutRule {
+    CutKind kind;
+    int words, rows;  // of a tile at most; a row of more words is an item of its own
+};
+constexpr int kCutChunk = 4096;  // a new tile starts at every multiple of this many rows (at 1,024 the
+                                 // part-filled tiles cost the batched product 2 %)
+CutRule csr_rule();              // csr.cu (variant 11)
+CutRule split_rule();            // split.cu (variant 14 and its batch)
+CutRule multi_rule();            // multi.cu
+packsell_status plan_items(Matrix &A, cudaStream_t s);  // all three lists of a matrix
+// The same cut on the host (a batch's lists), from the row offsets `off` of n
+// rows: push(base, r0, meta) receives each item in row order.
+template <typename Push>
+void cut_rows(const CutRule &rule, const int64_t *off, int n, Push push) {
+    int r = 0;
+    while (r < n) {
+        const int end = std::min({n, (r / kCutChunk + 1) * kCutChunk, r + rule.rows});
+        int t = r;
+        while (t < end && off[t + 1] - off[r] <= rule.words) ++t;
+        const int64_t w = t > r ? off[t] - off[r] : off[r + 1] - off[r];
+        push((long long)off[r], r,
+             t > r ? ((t - r) << 16) | (int)w : -(int)std::min<int64_t>(w, INT32_MAX));
+        r = std::max(t, r + 1);
+    }
+}
 SplitMat split_mat(const Matrix &A, const float *X, int64_t ldx, float *Y, int64_t ldy, int k);
 void multi_items_append(const int64_t *off, int64_t n, int mat, std::vector<MultiItem> &items);
 void multi_items_order(std::vector<MultiItem> &items);
-packsell_status multi_plan(Matrix &A, cudaStream_t s);
 void multi_plan_free(Matrix &A, const Release &rel);
 packsell_status launch_multi(const SplitMat &single, const SplitMat *mats, const MultiItem *items,
                              int nitems, int k, bool vec, cudaStream_t s);
 
 // split.cu
-packsell_status plan_split(Matrix &A, cudaStream_t s);
 void split_plan_free(Matrix &A, const Release &rel);
-packsell_status split_items_append(const int64_t *off, int64_t n, int mat,
-                                   std::vector<MultiItem> &items);
-packsell_status launch_split_batch(const SplitMat *mats, const MultiItem *items, int nitems,
+void split_items_append(const int64_t *off, int64_t n, int mat, std::vector<MultiItem> &items);
+packsell_status launch_split_batch(const SplitMat *mats, const MultiItem *items, int nitems, int nlong,
                                    bool sorted, cudaStream_t s);
 packsell_status launch_split(const Matrix &A, const void *perm, int pb, const float *x, float *y,
                              cudaStream_t s);

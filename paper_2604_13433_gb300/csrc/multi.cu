@@ -761,30 +761,13 @@ SplitMat split_mat(const Matrix &A, const float *X, int64_t ldx, float *Y, int64
     return M;
 }
 
-// Items of one C = 1 matrix from its host row offsets: consecutive rows of at
-// most MCT words grouped while they hold at most MCT words and MR_MAX rows;
-// a row of more words is an item of its own.
+CutRule multi_rule() { return CutRule{CUT_MULTI, MCT, MR_MAX}; }
+
+// Items of one C = 1 matrix of a batch from its host row offsets.
 void multi_items_append(const int64_t *off, int64_t n, int mat, std::vector<MultiItem> &items) {
-    auto tile = [&](int a, int b) {
-        items.push_back(MultiItem{(long long)off[a], a, ((b - a) << 16) | (int)(off[b] - off[a]), mat,
-                                  0, 0, 0});
-    };
-    int r0 = 0;
-    for (int r = 0; r < (int)n; ++r) {
-        const int64_t w = off[r + 1] - off[r];
-        if (w > MCT) {
-            if (r > r0) tile(r0, r);
-            items.push_back(MultiItem{(long long)off[r], r, -(int)std::min<int64_t>(w, INT32_MAX), mat,
-                                      0, 0, 0});
-            r0 = r + 1;
-            continue;
-        }
-        if (off[r + 1] - off[r0] > MCT || r + 1 - r0 > MR_MAX) {
-            tile(r0, r);
-            r0 = r;
-        }
-    }
-    if ((int)n > r0) tile(r0, (int)n);
+    cut_rows(multi_rule(), off, (int)n, [&](long long b, int r0, int meta) {
+        items.push_back(MultiItem{b, r0, meta, mat, 0, 0, 0});
+    });
 }
 
 // long rows first, longest first (the longest serial paths start first)
@@ -800,25 +783,6 @@ void multi_plan_free(Matrix &A, const Release &rel) {
     rel(A.multi_items);
     A.multi_items = nullptr;
     A.multi_nitems = 0;
-}
-
-packsell_status multi_plan(Matrix &A, cudaStream_t s) {
-    if (!is_packed(A.p.format) || A.p.C != 1 || A.n == 0) return PACKSELL_OK;
-    std::vector<int64_t> off((size_t)A.n + 1);
-    PS_CUDA(cudaMemcpyAsync(off.data(), A.offset, sizeof(int64_t) * (A.n + 1),
-                            cudaMemcpyDeviceToHost, s));
-    PS_CUDA(cudaStreamSynchronize(s));
-    std::vector<MultiItem> items;
-    items.reserve((size_t)(A.n_words / MCT + A.n / MR_MAX + 16));
-    multi_items_append(off.data(), A.n, 0, items);
-    multi_items_order(items);
-    if (items.size() >= (size_t)INT32_MAX) return fail(PACKSELL_ERR_RANGE, "multi_plan: too many items");
-    PS_CUDA(pool_get(&A.multi_items, sizeof(MultiItem) * items.size(), s));
-    PS_CUDA(cudaMemcpyAsync(A.multi_items, items.data(), sizeof(MultiItem) * items.size(),
-                            cudaMemcpyHostToDevice, s));
-    PS_CUDA(cudaStreamSynchronize(s));
-    A.multi_nitems = (int)items.size();
-    return PACKSELL_OK;
 }
 
 packsell_status launch_multi(const SplitMat &single, const SplitMat *mats, const MultiItem *items,

@@ -1099,11 +1099,7 @@ packsell_status plan_spmv(Matrix &A, cudaStream_t s) {
     }
     A.auto_variant = 1;
     if (is_packed(A.p.format) && A.p.C == 1 && A.n > 0 && A.n < INT32_MAX) {
-        packsell_status st = plan_csr(A, s);
-        if (st != PACKSELL_OK) return st;
-        st = plan_split(A, s);
-        if (st != PACKSELL_OK) return st;
-        st = multi_plan(A, s);
+        const packsell_status st = plan_items(A, s);
         if (st != PACKSELL_OK) return st;
         // untuned default for CSR order: the split-row kernel (all lanes busy
         // on rows of any length); variant 11 keeps the stored-order chain

@@ -74,3 +74,38 @@ def test_encode_on_streams_reuses_memory():
         if k >= 6:
             assert_same_encoding(A, enc)
         del A
+
+
+@pytest.mark.parametrize("n", [1, 255, 4095, 4096, 4097, 9000])
+@pytest.mark.parametrize("kind", ["short", "zipf", "near", "empty"])
+def test_csr_order_items_cover_the_rows(n, kind):
+    """CSR-order products over matrices whose items are cut at the edges of the
+    device cut's chunks and tiles (rows at the tile limits of the three kernels,
+    long rows, runs of empty rows): variant 11 gives the bits of the
+    thread-per-row kernel, variant 14 and the SpMM stay within gamma_w, and a
+    batch of the matrix gives variant 14's bits."""
+    need_gpu()
+    ps = P()
+    rng = np.random.default_rng(n)
+    lengths = {"short": rng.integers(0, 3, n), "zipf": np.minimum(rng.zipf(2.0, n), 900),
+               "near": rng.choice([1, 124, 125, 126, 252, 253, 254, 256, 257], n, p=[0.92] + [0.01] * 8),
+               "empty": np.where(rng.random(n) < 0.999, 0, 700)}[kind]
+    csr = _matrix([int(v) for v in lengths], 1000, seed=n + 1)
+    A = ps.packsell_encode_csr(csr, C=1, sigma=1)
+    deq = O.encode(csr, C=1, sigma=1, D=15, fmt=FMT["fp16"]).deq
+    x = I.uniform(csr.m, seed=2)
+    y = {}
+    for v in (1, 11, 14):
+        ps.packsell_set_spmv_variant(A, v)
+        y[v] = ps.packsell_spmv(A, dev(x))
+    assert torch.equal(y[1], y[11])
+    ref = O.csr_spmv_f64(csr, deq, x.astype(np.float64))
+    u = 2.0 ** -24
+    w = 2.0 * csr.row_lengths() + 1
+    tol = w * u / (1 - w * u) * O.csr_spmv_f64(csr, np.abs(deq), np.abs(x).astype(np.float64))
+    assert np.all(np.abs(y[14].cpu().numpy() - ref) <= tol)
+    X = dev(np.repeat(x[:, None], 20, 1))
+    assert np.all(np.abs(ps.packsell_spmm(A, X).cpu().numpy() - ref[:, None]) <= tol[:, None])
+    out = torch.full((csr.n,), -7.0, device="cuda")
+    ps.packsell_batch_spmv(ps.packsell_batch_create([A], [dev(x)], [out]))
+    assert torch.equal(out, y[14])
