@@ -342,6 +342,10 @@ packsell_status packsell_import(const void *h_blob, size_t bytes, void *stream,
     if (st != PACKSELL_OK) return bail(st);
     st = plan_spmv(*A, s);
     if (st != PACKSELL_OK) return bail(st);
+    // the plan's kernels are done on return: the matrix may be used on any
+    // stream, and products may read it before they wait on their stream
+    if (cudaStreamSynchronize(s) != cudaSuccess)
+        return bail(fail(PACKSELL_ERR_CUDA, "packsell_import: synchronize"));
     *out = reinterpret_cast<packsell_matrix *>(A);
     return PACKSELL_OK;
 }

@@ -109,3 +109,29 @@ def test_csr_order_items_cover_the_rows(n, kind):
     out = torch.full((csr.n,), -7.0, device="cuda")
     ps.packsell_batch_spmv(ps.packsell_batch_create([A], [dev(x)], [out]))
     assert torch.equal(out, y[14])
+
+
+@pytest.mark.parametrize("C,variants", [(1, (1, 11, 14)), (32, (1, 4, 9, 13))])
+def test_import_is_complete_on_return(C, variants):
+    """A matrix imported on one stream may be used on another at once: the
+    launch plans are finished when the call returns."""
+    need_gpu()
+    ps = P()
+    rng = np.random.default_rng(C)
+    csr = _matrix([int(v) for v in np.minimum(rng.zipf(2.0, 30000), 300)], 5000, seed=5)
+    A = ps.packsell_encode_csr(csr, C=C, sigma=1)
+    x = dev(I.uniform(csr.m, seed=6))
+    blob = ps.packsell_export(A)
+    s, t = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for v in variants:
+        ps.packsell_set_spmv_variant(A, v)
+        want = ps.packsell_spmv(A, x)
+        torch.cuda.synchronize()
+        B = ps.packsell_import(blob, stream=s)
+        assert s.query()
+        ps.packsell_set_spmv_variant(B, v)
+        with torch.cuda.stream(t):
+            y = ps.packsell_spmv(B, x)
+        t.synchronize()
+        assert torch.equal(y, want)
