@@ -196,7 +196,7 @@ template <typename Push>
 void cut_rows(const CutRule &rule, const int64_t *off, int n, Push push) {
     int r = 0;
     while (r < n) {
-        const int end = std::min({n, (r / kCutChunk + 1) * kCutChunk, r + rule.rows});
+        const int end = r + std::min({n - r, kCutChunk - r % kCutChunk, rule.rows});
         int t = r;
         while (t < end && off[t + 1] - off[r] <= rule.words) ++t;
         const int64_t w = t > r ? off[t] - off[r] : off[r + 1] - off[r];

@@ -26,7 +26,7 @@ struct CutArgs {
     CutRule rule[kPlans];
     int *tiles[kPlans];    // per chunk: tiles, then (after the scan) those before it
     int *bucket[kPlans];   // long rows per bucket, then the bucket's next place
-    int *totals;           // per plan: long rows, items
+    int *totals;           // per plan: long rows, items; then whether a row has INT32_MAX words or more
     void *items[kPlans];
     int n, chunks;
 };
@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(IW * 32) k_cut_items(CutArgs a, const int64_t 
     const int chunk = blockIdx.x * IW + (threadIdx.x >> 5);
     if (chunk >= a.chunks) return;
     const CutRule rule = a.rule[plan];
-    const int end = min(a.n, (chunk + 1) * kCutChunk);
     int r = chunk * kCutChunk;
+    const int end = r + min(a.n - r, kCutChunk);
     int tiles = FILL ? a.tiles[plan][chunk] : 0;
     while (r < end) {
         const long long o = off[r];
@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(IW * 32) k_cut_items(CutArgs a, const int64_t 
             if (lane == 0) {
                 const int at = atomicAdd(a.bucket[plan] + bucket_of(w), 1);
                 if (FILL) put(a, plan, at, o, r, 0, w);
+                else if (w >= INT32_MAX) a.totals[2 * kPlans] = 1;
             }
             r += 1;
         } else {
@@ -140,11 +141,11 @@ packsell_status plan_items(Matrix &A, cudaStream_t s) {
     CutArgs a{};
     a.n = (int)A.n;
     a.chunks = (int)((A.n + kCutChunk - 1) / kCutChunk);
-    const size_t ints = kPlans * ((size_t)a.chunks + kBuckets + 2);
-    int *mem = nullptr, h[2 * kPlans] = {};
+    const size_t ints = kPlans * ((size_t)a.chunks + kBuckets + 2) + 1;
+    int *mem = nullptr, h[2 * kPlans + 1] = {};
     PS_CUDA(pool_get(&mem, sizeof(int) * ints, s));
     a.totals = mem;
-    int *at = mem + 2 * kPlans;
+    int *at = mem + 2 * kPlans + 1;
     for (int p = 0; p < kPlans; ++p) {
         a.rule[p] = rules[p];
         a.bucket[p] = at;
@@ -155,7 +156,7 @@ packsell_status plan_items(Matrix &A, cudaStream_t s) {
         at += a.chunks;
     }
     const dim3 grid((a.chunks + IW - 1) / IW, kPlans);
-    cudaError_t e = cudaMemsetAsync(mem, 0, sizeof(int) * (2 + kBuckets) * kPlans, s);
+    cudaError_t e = cudaMemsetAsync(mem, 0, sizeof(int) * ((2 + kBuckets) * kPlans + 1), s);
     if (e == cudaSuccess) {
         k_cut_items<false><<<grid, IW * 32, 0, s>>>(a, A.offset);
         k_cut_scan<<<kPlans, 1024, 0, s>>>(a);
@@ -163,6 +164,10 @@ packsell_status plan_items(Matrix &A, cudaStream_t s) {
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, a.totals, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && h[2 * kPlans]) {
+        pool_put(mem, s);
+        return fail(PACKSELL_ERR_RANGE, "split-row plan: row too long");
+    }
     for (int p = 0; p < kPlans && e == cudaSuccess; ++p) {
         e = pool_get(out[p], item_bytes[p] * (size_t)h[2 * p + 1], s);
         a.items[p] = *out[p];
