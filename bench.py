@@ -405,10 +405,10 @@ def spmm_bytes(A, k):
 
 def spmm_kernel(C, k):
     """The kernel packsell_spmm runs for a C-row-slice matrix and k > 1 columns
-    (16-byte-aligned X and Y with k % 4 == 0)."""
+    (32-byte-aligned X and Y with k % 4 == 0, slices of at most 48 words when C = 32)."""
     if C == 1:
         return "k_split_rows" if k > 16 else "k_split_multi"
-    return "k_spmm_packed"
+    return "k_spmm_wide" if C == 32 and k % 8 == 0 else "k_spmm_packed"
 
 
 def irregular_section(ps, torch, dev, K, W, peak, n_rows=4194304):

@@ -760,7 +760,8 @@ void packsell_f3r_opts_default(packsell_f3r_opts *o);
  * inner_iters = layer-3 steps (iters * m2 * m3), relres = the last outer
  * estimate, relres_true, seconds (device time). Allocates its workspace
  * (stream-ordered) and SYNCHRONISES. Errors: INVALID_ARG, NO_MEMORY, CUDA,
- * NOT_CONVERGED (x holds the last iterate), BREAKDOWN (non-finite residual). */
+ * NOT_CONVERGED (x holds the last iterate), BREAKDOWN (non-finite residual),
+ * TIMEOUT (a grid-wide wait of a cooperative kernel ran out). */
 packsell_status packsell_f3r(const packsell_matrix *A_outer, const packsell_matrix *A_mid,
                              const packsell_matrix *A_low, const double *b, double *x,
                              const packsell_f3r_opts *opts, packsell_solve_result *result,
