@@ -62,7 +62,8 @@ __device__ __forceinline__ long long dummies_of(long long d, long long lim, int 
 // lane searches for the row of its element. A thread per row read its
 // columns a row length apart from its neighbours', twice (check, then
 // count), and sent two atomics per warp to two addresses (1.7 ns each, one
-// after another): 90 us on the 27-point 97 x 96 x 95 matrix (23.4M nonzeros).
+// after another): 90 us on the 27-point 97 x 96 x 95 matrix (23.4M nonzeros),
+// now 76 us (both under ncu, cold caches); the instruction rate bounds it.
 constexpr int SCAN_W = 8;  // warps per block
 
 __global__ void __launch_bounds__(SCAN_W * 32)
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(TPB)
 // row has fewer than 2^16 words, w and the position go into one 32-bit key
 // (w << 16 | 65535 - t: all keys differ, and the rank is the number of larger
 // ones), compared four at a time: two instructions per pair where the general
-// form takes five (47 us for 885,000 rows at sigma = 256).
+// form takes five (47 -> 32 us for 885,000 rows at sigma = 256).
 constexpr int SORT_TILE = 4096;
 
 __global__ void k_sigma_sort(int n, int sigma, const int32_t *__restrict__ words, void *perm,
@@ -554,7 +555,8 @@ packsell_status scan_exclusive(const int64_t *in, int64_t *out, int64_t S, cudaS
 // there, and the lanes' words of one j go out together. Quantising here
 // instead of in a pass of its own saves writing and reading the fields: 59 +
 // 69 us for the two passes on the 27-point 97 x 96 x 95 matrix (23.4M
-// nonzeros, 281 MB in and out). Rounds of 32 entries; of 8 where the rows
+// nonzeros, 281 MB in and out), now 79 us for one (3.6 TB/s; bound by the
+// copies' latency). Rounds of 32 entries; of 8 where the rows
 // have no more on average (fewer idle lanes per copy).
 // Rows past n (phantom rows of the last slice) get padding only.
 constexpr int SC_W = 4;  // warps per block

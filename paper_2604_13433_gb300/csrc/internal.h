@@ -184,8 +184,7 @@ struct CutRule {
     CutKind kind;
     int words, rows;  // of a tile at most; a row of more words is an item of its own
 };
-constexpr int kCutChunk = 4096;  // a new tile starts at every multiple of this many rows (at 1,024 the
-                                 // part-filled tiles cost the batched product 2 %)
+constexpr int kCutChunk = 4096;  // a chunk of this many rows without a long row starts a tile of its own
 CutRule csr_rule();              // csr.cu (variant 11)
 CutRule split_rule();            // split.cu (variant 14 and its batch)
 CutRule multi_rule();            // multi.cu
@@ -194,9 +193,17 @@ packsell_status plan_items(Matrix &A, cudaStream_t s);  // all three lists of a 
 // rows: push(base, r0, meta) receives each item in row order.
 template <typename Push>
 void cut_rows(const CutRule &rule, const int64_t *off, int n, Push push) {
+    auto any_long = [&](int c0) {
+        const int c1 = c0 + std::min(n - c0, kCutChunk);
+        for (int q = c0; q < c1; ++q)
+            if (off[q + 1] - off[q] > rule.words) return true;
+        return false;
+    };
     int r = 0;
     while (r < n) {
-        const int end = r + std::min({n - r, kCutChunk - r % kCutChunk, rule.rows});
+        const int c0 = r - r % kCutChunk;
+        int end = r + std::min(n - r, rule.rows);
+        if (end - c0 > kCutChunk && !any_long(c0 + kCutChunk)) end = c0 + kCutChunk;
         int t = r;
         while (t < end && off[t + 1] - off[r] <= rule.words) ++t;
         const int64_t w = t > r ? off[t] - off[r] : off[r + 1] - off[r];

@@ -4,10 +4,15 @@
 // long rows, long rows first and the longest of them early (they are the
 // longest serial paths), tiles in row order. The rule is one (struct
 // CutRule): from row r0 a tile takes the most rows that hold at most `words`
-// words and are at most `rows`; a row of more words is an item of its own;
-// and every kCutChunk rows a new tile starts, so that chunks can be cut
-// independently, one warp each. (On the host, from a copy of the row offsets,
-// the three lists of a 1.4M-row matrix took about 20 ms of its encoding.)
+// words and are at most `rows`; a row of more words is an item of its own. So
+// a tile starts behind every long row whatever was cut before it, and the rows
+// are cut in parallel, one warp per chunk of kCutChunk rows: from behind the
+// first long row of its chunk to behind the first of the next. Where a chunk
+// has no long row a tile starts at its first row instead. (A tile started at
+// every chunk gave 0.5 to 1 % more items, which cost variant 14 up to 4.5 %
+// where the last round of its warps became one longer: 28.7 -> 30.0 us on a
+// power-law matrix of 1M rows. On the host, from a copy of the row offsets, the
+// three lists of a 1.4M-row matrix took about 20 ms of its encoding.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -48,6 +53,28 @@ __device__ __forceinline__ void put(const CutArgs &a, int plan, int at, long lon
         ((MultiItem *)a.items[plan])[at] = MultiItem{base, r0, meta, 0, 0, 0, 0};
 }
 
+// The first row that a chunk's warp cuts: behind the chunk's first long row, or
+// the chunk's first row where it has none (n past the last chunk).
+__device__ int cut_start(const CutArgs &a, int words, int chunk, const int64_t *__restrict__ off) {
+    if (chunk == 0) return 0;
+    if (chunk >= a.chunks) return a.n;
+    const int lane = threadIdx.x & 31, r0 = chunk * kCutChunk, len = min(a.n - r0, kCutChunk);
+    for (int t0 = 0; t0 < len; t0 += 128) {
+        int64_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int t = t0 + 32 * q + lane;
+            w[q] = t < len ? off[r0 + t + 1] - off[r0 + t] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const unsigned hit = __ballot_sync(0xffffffffu, w[q] > words);
+            if (hit) return r0 + t0 + 32 * q + __ffs(hit);
+        }
+    }
+    return r0;
+}
+
 // One warp per chunk of rows: the number of rows of the next tile by two
 // rounds of 32 offset reads (eight rows apart, then one).
 template <bool FILL>
@@ -56,8 +83,8 @@ __global__ void __launch_bounds__(IW * 32) k_cut_items(CutArgs a, const int64_t 
     const int chunk = blockIdx.x * IW + (threadIdx.x >> 5);
     if (chunk >= a.chunks) return;
     const CutRule rule = a.rule[plan];
-    int r = chunk * kCutChunk;
-    const int end = r + min(a.n - r, kCutChunk);
+    int r = cut_start(a, rule.words, chunk, off);
+    const int end = cut_start(a, rule.words, chunk + 1, off);
     int tiles = FILL ? a.tiles[plan][chunk] : 0;
     while (r < end) {
         const long long o = off[r];
