@@ -169,7 +169,13 @@ __device__ __forceinline__ bool uses_second(int fin) {
     return fin == FIN_RZ_BETA_RR || fin == FIN_OUTER_ALPHA || fin == FIN_BB_RR;
 }
 
-// Every thread of every block calls this once with its contributions.
+// Every thread of every block calls this once with its contributions. BATCHED:
+// the last block's threads load six partials at a time (one by one they cost
+// the tail of the FP32 inner kernels a trip to the L2 each: 6 us with 912 blocks
+// and two sums). The FP64 kernels take them one by one: the registers of the
+// six cost them more than the tail gives (FP64 PCG on 7-point 256^3 0.827 s
+// against 0.852 s; the inner FP32 solves 0.411 s against 0.408 s, E8M11).
+template <bool BATCHED = true>
 __device__ __forceinline__ void reduce_publish(const Red &r, double v1, double v2) {
     __shared__ bool last;
     const bool two = uses_second(r.fin);
@@ -183,22 +189,27 @@ __device__ __forceinline__ void reduce_publish(const Red &r, double v1, double v
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // the partials of a thread load together (added one by one they cost the
-    // kernel's tail a trip to the L2 each: 6 us with 912 blocks and two sums)
-    constexpr int U = 6;
     double a = 0.0, b = 0.0;
-    for (unsigned q0 = threadIdx.x; q0 < gridDim.x; q0 += U * blockDim.x) {
-        double va[U], vb[U];
+    if (BATCHED) {
+        constexpr int U = 6;
+        for (unsigned q0 = threadIdx.x; q0 < gridDim.x; q0 += U * blockDim.x) {
+            double va[U], vb[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const unsigned q = q0 + u * blockDim.x;
-            va[u] = q < gridDim.x ? ((volatile double *)r.partials)[2 * q] : 0.0;
-            vb[u] = two && q < gridDim.x ? ((volatile double *)r.partials)[2 * q + 1] : 0.0;
+            for (int u = 0; u < U; ++u) {
+                const unsigned q = q0 + u * blockDim.x;
+                va[u] = q < gridDim.x ? ((volatile double *)r.partials)[2 * q] : 0.0;
+                vb[u] = two && q < gridDim.x ? ((volatile double *)r.partials)[2 * q + 1] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                a += va[u];
+                if (two) b += vb[u];
+            }
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            a += va[u];
-            if (two) b += vb[u];
+    } else {
+        for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
+            a += ((volatile double *)r.partials)[2 * q];
+            b += ((volatile double *)r.partials)[2 * q + 1];
         }
     }
     block_sum2(a, b, two);

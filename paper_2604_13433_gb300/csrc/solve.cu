@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(VTPB)
         bb += bi * bi;
         rr += ri * ri;
     }
-    reduce_publish(red, red.fin == FIN_RT ? rr : bb, rr);
+    reduce_publish<false>(red, red.fin == FIN_RT ? rr : bb, rr);
 }
 
 // PCG start (type T): z = M r, p = z, s1 = r.z
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(VTPB)
         p[i] = z;
         rz = fma(r[i], z, rz);
     }
-    reduce_publish(red, (double)rz, 0.0);
+    reduce_publish<sizeof(T) == 4>(red, (double)rz, 0.0);
 }
 
 // Inner PCG start: r_in = r / ||r|| (rounded to FP32), x_in = 0, p = M r_in.
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(VTPB)
     } else {
         PS_FOR(i, n) one(i);
     }
-    reduce_publish(red, (double)rz, (double)rr);
+    reduce_publish<sizeof(T) == 4>(red, (double)rz, (double)rr);
 }
 
 // Direction update. MODE 0: p = M r + beta p. MODE 1: first x += alpha p
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(VTPB)
         z[i] = zi;
         zq += zi * q[i];
     }
-    reduce_publish(red, zq, 0.0);
+    reduce_publish<false>(red, zq, 0.0);
 }
 
 // Outer: p = z - beta_o p (beta_o = 0 right after a (re)start)
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(VTPB)
         r[i] = ri;
         rr += ri * ri;
     }
-    reduce_publish(red, rr, 0.0);
+    reduce_publish<false>(red, rr, 0.0);
 }
 
 __global__ void k_f64_to_f32(int64_t n, const double *__restrict__ a, float *__restrict__ b) {

@@ -891,7 +891,7 @@ __device__ __forceinline__ void sell_rows(int n, int C, int sigma,
             if (b) d2 = fma(x[io], b[io], d2);
         }
     }
-    if (DOT) reduce_publish(red, (double)d1, (double)d2);
+    if (DOT) reduce_publish<sizeof(T) == 4>(red, (double)d1, (double)d2);
 }
 
 template <typename T, bool DOT = false, bool PDL = false>

@@ -76,7 +76,7 @@ __device__ __forceinline__ void w64_rows(int n, int C, int sigma, long long k_le
             if (b) d2 = fma(x[io], b[io], d2);
         }
     }
-    if (DOT) reduce_publish(red, d1, d2);
+    if (DOT) reduce_publish<false>(red, d1, d2);
 }
 
 __global__ void __launch_bounds__(TPB)
