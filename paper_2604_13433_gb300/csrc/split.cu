@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(SW * 32, 4)
 // in matrix and row order, go to the blocks in contiguous runs, so that a block
 // reads few matrix descriptors and gathers from one part of an x at a time.
 // Within the block the warps draw tickets: a warp with a long row takes fewer
-// tiles. Batch of 256 power-law matrices: 132.5 -> 130.8 us against items w,
+// tiles. Batch of 256 power-law matrices: 133.0 -> 130.0 us against items w,
 // w + W, w + 2W, ... for warp w. (One matrix of 4M rows: 84.5 -> 86.1 us, so
 // variant 14 keeps that order.)
 struct BlockItems {
