@@ -251,8 +251,11 @@ packsell_status packsell_permute_csr(int64_t n, const int64_t *rowptr, const int
                                      const void *val, int32_t val_is_f64, const int32_t *perm,
                                      int64_t *out_rowptr, int32_t *out_col, void *out_val);
 
-/* Free the matrix (synchronises the device first). NULL is accepted.
- * Housekeeping with no counterpart in the paper. */
+/* Free the matrix (synchronises the matrix's device first, whichever device is
+ * current). Where the device cannot be synchronised, as while one of its
+ * streams is being captured, the memory is given back by a later destroy on
+ * that device or when an allocation runs out. NULL is accepted. Housekeeping
+ * with no counterpart in the paper. */
 packsell_status packsell_destroy(packsell_matrix *A);
 
 packsell_status packsell_get_info(const packsell_matrix *A, packsell_info *info);

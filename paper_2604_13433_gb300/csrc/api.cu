@@ -34,8 +34,6 @@ int64_t matrix_bytes(const Matrix &A) {
     return b;
 }
 
-void destroy_matrix(Matrix *A);
-
 // Readers of the bounds-check counters, one per translation unit (registered
 // while the library loads; empty in the regular build).
 static std::vector<ChecksReader> &checks_readers() {

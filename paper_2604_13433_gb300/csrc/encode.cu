@@ -25,6 +25,7 @@
 
 #include "device.cuh"
 #include "internal.h"
+#include "release.h"
 
 namespace packsell {
 namespace {
@@ -941,7 +942,7 @@ packsell_status encode_impl(const packsell_params &p, int64_t n, int64_t m, int6
     A->perm_bytes = perm_bytes;
     cudaGetDevice(&A->device);
     auto bail = [&](packsell_status st) {
-        free_matrix_arrays(A, Release{true, s});  // every use so far is on s
+        free_matrix_arrays(A, Release{s});  // every use so far is on s
         delete A;
         return st;
     };
@@ -1150,16 +1151,44 @@ packsell_status encode_impl(const packsell_params &p, int64_t n, int64_t m, int6
     return PACKSELL_OK;
 }
 
+namespace {
+
+struct CudaRt {
+    bool device(int *dev) { return ok(cudaGetDevice(dev)); }
+    bool set_device(int dev) { return ok(cudaSetDevice(dev)); }
+    bool wait() { return ok(cudaDeviceSynchronize()); }
+    void give_back(Matrix *A) {
+        free_matrix_arrays(A, Release{cudaStreamPerThread});
+        delete A;
+    }
+    // a failed call's error must not be found by the next launch check
+    static bool ok(cudaError_t e) {
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess;
+    }
+};
+
+Retired<Matrix, CudaRt> &retired() {
+    static Retired<Matrix, CudaRt> r;
+    return r;
+}
+
+}  // namespace
+
+// products may still run on any stream of the matrix's device (no host memory
+// for the list: the matrix is leaked)
 void destroy_matrix(Matrix *A) {
-    if (!A) return;
-    // products may still run on any stream: the arrays go back to the pool
-    // once the device has finished; where that cannot be waited for here (the
-    // matrix of another device, a capture in progress) cudaFree waits itself
-    int dev = -1;
-    const bool idle = cudaGetDevice(&dev) == cudaSuccess && dev == A->device &&
-                      cudaDeviceSynchronize() == cudaSuccess;
-    free_matrix_arrays(A, Release{idle, cudaStreamPerThread});
-    delete A;
+    try {
+        if (A) retired().retire(A->device, A, CudaRt{});
+    } catch (...) {
+    }
+}
+
+void flush_destroyed(int dev) {
+    try {
+        retired().flush(dev, CudaRt{});
+    } catch (...) {
+    }
 }
 
 // ---- validation of imported matrices ----

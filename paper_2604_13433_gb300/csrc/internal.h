@@ -100,7 +100,10 @@ packsell_status encode_impl(const packsell_params &p, int64_t n, int64_t m, int6
                             const int64_t *rowptr, const int32_t *col, const void *val,
                             int val_is_f64, cudaStream_t s, Matrix **out);
 packsell_status validate_impl(const Matrix &A, cudaStream_t s, const char *what);
+// A's memory goes back once A's device has finished (release.h), at once or in
+// a later call; flush_destroyed gives back what waits on `dev`
 void destroy_matrix(Matrix *A);
+void flush_destroyed(int dev);
 
 // pool.cu: stream-ordered device memory from the library's pool (one per
 // device). pool_get: usable by work on `s`, and by any stream once `s` has
@@ -112,17 +115,11 @@ cudaError_t pool_get(T **p, size_t bytes, cudaStream_t s) {
 }
 void pool_put(void *p, cudaStream_t s);
 
-// How an object's arrays are given back: in the order of a stream (every use
-// of them lies before on that stream, or the device has been synchronised),
-// or by cudaFree, which waits for the device.
+// How an object's arrays are given back: in the order of a stream. Every use of
+// them lies before on that stream, or the device has been synchronised.
 struct Release {
-    bool ordered;
     cudaStream_t s;
-    void operator()(void *p) const {
-        if (!p) return;
-        if (ordered) pool_put(p, s);
-        else cudaFree(p);
-    }
+    void operator()(void *p) const { pool_put(p, s); }
 };
 packsell_status quantize_impl(int fmt, int D, int64_t n, const void *val, int is64, uint32_t *field,
                               int64_t *bad_index, cudaStream_t s);

@@ -65,6 +65,7 @@ cudaError_t pool_get(void **p, size_t bytes, cudaStream_t s) {
     e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
+        flush_destroyed(dev);
         cudaStreamSynchronize(s);
         cudaMemPoolTrimTo(pool, 0);
         e = cudaMallocFromPoolAsync(p, bytes, pool, s);
@@ -78,8 +79,11 @@ void pool_put(void *p, cudaStream_t s) {
     int dev = 0;
     cudaMemPool_t pool;
     if (cudaFreeAsync(p, s) != cudaSuccess) {
+        // cudaFree of pool memory waits for nothing: only after the device has
+        // finished, or not at all
         cudaGetLastError();
-        cudaFree(p);  // any allocation; waits for the device
+        if (cudaDeviceSynchronize() == cudaSuccess) cudaFree(p);
+        cudaGetLastError();
     }
     if (cudaGetDevice(&dev) == cudaSuccess && pool_of(dev, &pool) == cudaSuccess) set_threshold(pool);
 }
