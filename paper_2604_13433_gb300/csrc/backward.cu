@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(BW * 32, 4)
     const float g = DX && live ? dy[dy_storage ? i : io] : 0.f;
     const float a = DV && live ? alpha * dy[io] : 0.f;
     long long q = DV && live ? rowptr[io] : 0;
+    const long long qend = DV && live ? rowptr[io + 1] : 0;  // (the bounds-check build's)
     for (int j0 = 0; j0 < w; j0 += BR) {
         uint32_t wd[BR];
 #pragma unroll
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(BW * 32, 4)
             int t = 0;
 #pragma unroll
             for (int u = 0; u < BR; ++u)
-                if (wd[u] & 1u) s_val[wl][lane * BS + t++] = a * xv[u];
+                if ((wd[u] & 1u) && PS_IN_RANGE(q + t, qend)) s_val[wl][lane * BS + t++] = a * xv[u];
             s_run[wl][lane] = RowRun{q, t, 0};
             q += t;
             __syncwarp();
