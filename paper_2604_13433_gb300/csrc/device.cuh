@@ -113,13 +113,49 @@ inline Decode make_decode(const Matrix &A) {
     return d;
 }
 
-// One word: add its delta to c; if it carries a value, gather x_c.
-template <int FMT>
+// Loads of vectors that the previous kernel of the stream may still be
+// writing when this kernel starts (launch_pdl, below). __ldg, and plain loads
+// through const __restrict__ pointers, are ld.global.nc: PTX allows them only
+// for memory that nothing writes while the kernel runs, so they may be moved
+// above griddepcontrol.wait and may hit a line that was cached before the
+// write. These are ordinary global loads, which the wait makes the
+// predecessor's writes visible to, and volatile asm, which stays behind it.
+__device__ __forceinline__ float ld_dep(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_dep(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half ld_dep(const __half *p) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
+}
+__device__ __forceinline__ float4 ld_dep(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_dep(const double2 *p) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+
+// One word: add its delta to c; if it carries a value, gather x_c (DEP: in a
+// kernel started by launch_pdl).
+template <int FMT, bool DEP = false>
 __device__ __forceinline__ void word_gather(uint32_t wd, Decode dc, const float *__restrict__ x,
                                             int &c, bool &f, float &xv) {
     f = (wd & 1u) != 0u;
     c += (int)((wd >> 1) & (f ? dc.dmask : 0x7fffffffu));
-    if (f) xv = PS_IN_RANGE(c, dc.xlen) ? __ldg(x + c) : 0.f;
+    if (f) xv = PS_IN_RANGE(c, dc.xlen) ? (DEP ? ld_dep(x + c) : __ldg(x + c)) : 0.f;
 }
 
 // The value a word carries (FP16 in the upper half, or E8MY bits).
@@ -140,12 +176,17 @@ __device__ __forceinline__ uint32_t ldg_stream(const uint32_t *p) { return __ldc
 // of its stream drains. grid_dep_sync first waits until that kernel has
 // completed and its memory is visible (at once when there is none), then
 // lets the next kernel of the stream be scheduled once every block of this
-// grid has passed the same point (or exited). Signalling only after the
-// wait keeps at most one kernel waiting ahead: signalled at block start, a
-// chain of persistent-grid solver kernels queued up on the SMs and slowed the
-// one running. The product kernels read only the matrix (complete when
-// encode or import returns, never written by a product) before the call,
-// and x, y and solver state after it.
+// grid has passed the same point (or exited). Every kernel signals only
+// after its wait, so that no more than two grids of a stream are ever in
+// flight and the one before them has completed: signalled at block start,
+// products in a row in a captured graph gave results that varied from run to
+// run, and a chain of persistent-grid solver kernels queued up on the SMs and
+// slowed the one running. A product of more blocks than fit at a time loses
+// nothing by it: its dependents can only be scheduled once its last wave has
+// started, long after its wait. The product kernels read only the matrix
+// (complete when encode or import returns, never written by a product) before
+// the wait, and x, y and solver state after it, by ld_dep or other loads that
+// the compiler does not take for read-only data.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -154,9 +195,6 @@ __device__ __forceinline__ void grid_dep_sync() {
     grid_dep_wait();
     grid_dep_launch();
 }
-// A grid that covers the rows once (more blocks than fit at a time) may
-// signal at block start instead: its dependents can then only be scheduled
-// once its last wave has started.
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t s,

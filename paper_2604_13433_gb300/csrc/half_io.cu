@@ -22,7 +22,6 @@ __global__ void __launch_bounds__(TPB)
                const int64_t *__restrict__ offset, const uint32_t *__restrict__ pack,
                const void *__restrict__ perm, int perm_bytes, Decode dc,
                const __half *__restrict__ x, __half *__restrict__ y) {
-    grid_dep_launch();  // one pass over the rows: signal at block start
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int k = i >> 5;
@@ -32,21 +31,21 @@ __global__ void __launch_bounds__(TPB)
     const int blk = sig_shift >= 0 ? (i >> sig_shift) << sig_shift : (i / sigma) * sigma;
     int c = (k_left < blk) ? (int)(blk - k_left) : 0;
     float t = 0.f;
-    if (w <= 0) grid_dep_wait();
+    if (w <= 0) grid_dep_sync();
     for (int j0 = 0; j0 < w; j0 += PF) {
         const int wr = w - j0;
         uint32_t wd[PF];
 #pragma unroll
         for (int u = 0; u < PF; ++u) wd[u] = (u < wr) ? ldg_stream(pp + (j0 + u) * 32) : 0u;
         // the first round's words load before the wait; x and y after it
-        if (j0 == 0) grid_dep_wait();
+        if (j0 == 0) grid_dep_sync();
         bool f[PF];
         float xv[PF];
 #pragma unroll
         for (int u = 0; u < PF; ++u) {
             f[u] = (wd[u] & 1u) != 0u;
             c += (int)((wd[u] >> 1) & (f[u] ? dc.dmask : 0x7fffffffu));
-            if (f[u]) xv[u] = PS_IN_RANGE(c, dc.xlen) ? __half2float(__ldg(x + c)) : 0.f;
+            if (f[u]) xv[u] = PS_IN_RANGE(c, dc.xlen) ? __half2float(ld_dep(x + c)) : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < PF; ++u)

@@ -116,10 +116,11 @@ __device__ __forceinline__ void stv(T *p, int64_t v, const T (&e)[V<T>::W]) {
 // FP64 rate is too low to spend per element) and the block and grid sums
 // are FP64. Without XUP the x update of the iteration is left to the next
 // direction kernel (k_pupdate, which reads p anyway), or to the final one.
+// No vector is __restrict__ here and below: the previous kernel may still be
+// writing it when this one starts (ld_dep in device.cuh says why).
 template <typename T, bool VEC, bool XUP>
 __global__ void __launch_bounds__(VTPB)
-    k_update(int64_t n, T *__restrict__ x, T *__restrict__ r, const T *__restrict__ p,
-             const T *__restrict__ q, const T *__restrict__ M, Red red) {
+    k_update(int64_t n, T *x, T *r, const T *p, const T *q, const T *M, Red red) {
     grid_dep_sync();  // launched by launch_pdl: everything it reads comes from earlier kernels
     if (red.sc->done) return;
     const T a = (T)red.sc->alpha;
@@ -182,13 +183,17 @@ __global__ void __launch_bounds__(VTPB)
 // the iteration's (alpha is not rewritten before the next product).
 template <typename T, bool VEC, int MODE>
 __global__ void __launch_bounds__(VTPB)
-    k_pupdate(int64_t n, const T *__restrict__ r, const T *__restrict__ M, T *__restrict__ p,
-              T *__restrict__ x, const SolveScalars *sc) {
+    k_pupdate(int64_t n, const T *r, const T *M, T *p, T *x, const SolveScalars *sc) {
     grid_dep_sync();  // launched by launch_pdl, as k_update
     if (sc->done) return;
     const T b = (T)sc->beta;
     const T a = (T)sc->alpha;
     constexpr bool XU = MODE != 0, PU = MODE != 2;
+    auto one = [&](int64_t i) {
+        const T pi = p[i];
+        if (XU) x[i] = fma(a, pi, x[i]);
+        if (PU) p[i] = fma(b, pi, M ? M[i] * r[i] : r[i]);
+    };
     if (VEC) {
         constexpr int W = V<T>::W;
         const int64_t nv = n / W, tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -225,18 +230,9 @@ __global__ void __launch_bounds__(VTPB)
                 }
             }
         }
-        for (int64_t i = nv * W + tid; i < n; i += st) {
-            if (XU) x[i] = fma(a, p[i], x[i]);
-            if (PU) p[i] = fma(b, p[i], M ? M[i] * r[i] : r[i]);
-        }
+        for (int64_t i = nv * W + tid; i < n; i += st) one(i);
     } else {
-        PS_FOR(i, n) {
-            if (XU) x[i] = fma(a, p[i], x[i]);
-            if (PU) {
-                const T z = M ? M[i] * r[i] : r[i];
-                p[i] = fma(b, p[i], z);
-            }
-        }
+        PS_FOR(i, n) one(i);
     }
 }
 

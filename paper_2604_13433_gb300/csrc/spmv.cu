@@ -80,7 +80,10 @@ __global__ void __launch_bounds__(TPB)
 // gathers. Words past the row's slice width are taken as 0 (padding).
 // One row of the prefetch kernels: returns the sum, sets the output index
 // (PERM: rows are written through the sigma permutation).
-template <int FMT, int PF, int C, bool PERM = true, bool EXIT = false, bool PDL = false>
+// PDL (launched by launch_pdl): waits for the previous kernel and, with SIGNAL,
+// lets the next one be scheduled.
+template <int FMT, int PF, int C, bool PERM = true, bool EXIT = false, bool PDL = false,
+          bool SIGNAL = PDL>
 __device__ __forceinline__ float prefetch_row(int i, int sigma, int sig_shift, long long k_left,
                                               const int64_t *__restrict__ offset,
                                               const uint32_t *__restrict__ pack,
@@ -93,7 +96,11 @@ __device__ __forceinline__ float prefetch_row(int i, int sigma, int sig_shift, l
     const int blk = sig_shift >= 0 ? (i >> sig_shift) << sig_shift : (i / sigma) * sigma;
     int c = (k_left < blk) ? (int)(blk - k_left) : 0;
     float t = 0.f;
-    if (PDL && w <= 0) grid_dep_wait();
+    auto dep = [] {
+        grid_dep_wait();
+        if (SIGNAL) grid_dep_launch();
+    };
+    if (PDL && w <= 0) dep();
     for (int j0 = 0; j0 < w; j0 += PF) {
         const int wr = w - j0;
         // loads predicated on the width; a word past it acts as padding
@@ -103,11 +110,11 @@ __device__ __forceinline__ float prefetch_row(int i, int sigma, int sig_shift, l
         // PDL: the matrix is complete before any product runs, so the first
         // round's words (and the offsets) load while the previous kernel of
         // the stream finishes; x and y are touched only after the wait
-        if (PDL && j0 == 0) grid_dep_wait();
+        if (PDL && j0 == 0) dep();
         bool f[PF];
         float xv[PF];
 #pragma unroll
-        for (int u = 0; u < PF; ++u) word_gather<FMT>(wd[u], dc, x, c, f[u], xv[u]);
+        for (int u = 0; u < PF; ++u) word_gather<FMT, PDL>(wd[u], dc, x, c, f[u], xv[u]);
 #pragma unroll
         for (int u = 0; u < PF; ++u)
             if (f[u]) t = fmaf(word_value<FMT>(wd[u], dc), xv[u], t);
@@ -133,11 +140,8 @@ struct Epilogue {
     float omega = 0.f;
 };
 
-// Volatile loads: the addresses are known before the kernel's wait on its
-// predecessor, and loads through const __restrict__ pointers may be moved
-// above that wait (they then read the vectors before they are written).
 __device__ __forceinline__ float epilogue(const Epilogue &e, const float *x, int io, float t) {
-    const float xi = *(const volatile float *)(x + io), ri = *(const volatile float *)(e.r + io);
+    const float xi = ld_dep(x + io), ri = ld_dep(e.r + io);
     return fmaf(e.omega, ri - t, xi);
 }
 
@@ -153,14 +157,11 @@ __global__ void __launch_bounds__(TPB, MINB)
                     const float *__restrict__ x, float *__restrict__ y, Red red = Red{},
                     Epilogue ep = Epilogue{}) {
     if (!DOT) {
-        // one pass over the rows: signal at block start. Not with an epilogue:
-        // there the next kernel of a captured graph is again a product launched
-        // this way, and two in a row that signal early gave wrong results
-        if (PDL && !EPI) grid_dep_launch();
+        // (the form with an epilogue sends no signal: it has not been measured with one)
         const int i = blockIdx.x * blockDim.x + threadIdx.x;
         if (i >= n) return;
         int io;
-        const float t = prefetch_row<FMT, PF, C, PERM, EXIT, PDL>(
+        const float t = prefetch_row<FMT, PF, C, PERM, EXIT, PDL, PDL && !EPI>(
             i, sigma, sig_shift, k_left, offset, pack, perm, perm_bytes, dc, x, io);
         y[io] = EPI ? epilogue(ep, x, io, t) : t;
         return;
@@ -184,13 +185,13 @@ __global__ void __launch_bounds__(TPB, MINB)
 // after it, before it decodes and gathers the current row: the word loads
 // of one row overlap the gathers of the previous one. Every slice must fit
 // one round (width <= PF <= 16). Same bits as the thread-per-row kernels.
-template <int FMT, int PF>
+template <int FMT, int PF, bool DEP>
 __device__ __forceinline__ void pipe_round(const uint32_t (&wd)[PF], Decode dc,
                                            const float *__restrict__ x, int &c, float &t) {
     bool f[PF];
     float xv[PF];
 #pragma unroll
-    for (int u = 0; u < PF; ++u) word_gather<FMT>(wd[u], dc, x, c, f[u], xv[u]);
+    for (int u = 0; u < PF; ++u) word_gather<FMT, DEP>(wd[u], dc, x, c, f[u], xv[u]);
 #pragma unroll
     for (int u = 0; u < PF; ++u)
         if (f[u]) t = fmaf(word_value<FMT>(wd[u], dc), xv[u], t);
@@ -241,12 +242,12 @@ __global__ void __launch_bounds__(TPB, MINB)
             const int blk = sig_shift >= 0 ? (i >> sig_shift) << sig_shift : (i / sigma) * sigma;
             int c = (k_left < blk) ? (int)(blk - k_left) : 0;
             float t = 0.f;
-            pipe_round<FMT, PF>(cur, dc, x, c, t);
+            pipe_round<FMT, PF, PDL>(cur, dc, x, c, t);
             int io = i;
             if (PERM) io = blk + (perm_bytes == 1 ? (int)((const uint8_t *)perm)[i]
                                                   : (int)((const uint16_t *)perm)[i]);
             y[io] = t;
-            if (DOT) d1 = fmaf(x[io], t, d1);
+            if (DOT) d1 = fmaf(PDL ? ld_dep(x + io) : x[io], t, d1);
             if (in >= n) break;
             i = in;
 #pragma unroll
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(TPB, MINB)
             }
             float xv[PF];
 #pragma unroll
-            for (int u = 0; u < PF; ++u) xv[u] = u < w ? __ldg(x + cc[u]) : 0.f;
+            for (int u = 0; u < PF; ++u) xv[u] = u < w ? ld_dep(x + cc[u]) : 0.f;
             float t = 0.f;
 #pragma unroll
             for (int u = 0; u < PF; ++u)
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(TPB, MINB)
                                             : (int)((const uint16_t *)perm)[i]);
             }
             y[io] = t;
-            d1 = fmaf(x[io], t, d1);
+            d1 = fmaf(ld_dep(x + io), t, d1);
             if (in >= n) break;
             i = in;
             w = wn;
@@ -464,7 +465,9 @@ packsell_status launch_prefetch(const Matrix &A, const void *perm, int pb, const
 // Variant 13: the kernel of variant 5 (rows run to the slice width) launched
 // with programmatic stream serialisation, so that its blocks are scheduled
 // while the previous kernel of the stream drains and load their first words
-// before they wait for it.
+// before they wait for it: 45.1 -> 41.6 us on the 27-point 128^3 matrix in
+// explicit order. The signal after the wait and the ordinary loads of x
+// (ld_dep), without which a chain of products is not safe, cost 0.3 us of it.
 template <int FMT, int PF, int MINB>
 packsell_status launch_prefetch_pdl(const Matrix &A, const void *perm, int pb, const float *x,
                                     float *y, cudaStream_t s) {
@@ -852,8 +855,8 @@ __device__ __forceinline__ void sell_rows(int n, int C, int sigma,
                                           const void *__restrict__ perm, int perm_bytes,
                                           const T *__restrict__ x, T *__restrict__ y,
                                           const T *__restrict__ b, Red red) {
+    auto ldx = [](const T *p) { return PDL ? ld_dep(p) : __ldg(p); };
     if (DOT && PDL) grid_dep_sync();  // the reducing form waits before it starts
-    if (!DOT && PDL) grid_dep_launch();  // one pass over the rows: signal at block start
     if (DOT && red.sc->done) return;  // solver converged: idle (grid-uniform)
     T d1 = 0, d2 = 0;  // per-thread sums in T; block and grid sums in FP64
     const int stride = DOT ? gridDim.x * blockDim.x : n;
@@ -865,7 +868,7 @@ __device__ __forceinline__ void sell_rows(int n, int C, int sigma,
         const int32_t *cp = col + s + l;
         T t = 0;
         int j = 0;
-        if (PDL && !DOT && w < UNROLL) grid_dep_wait();
+        if (PDL && !DOT && w < UNROLL) grid_dep_sync();
         for (; j + UNROLL <= w; j += UNROLL) {
             T v[UNROLL];
             int cc[UNROLL];
@@ -875,20 +878,21 @@ __device__ __forceinline__ void sell_rows(int n, int C, int sigma,
                 cc[u] = __ldcs(cp + (int64_t)(j + u) * C);
             }
             // every round (returns at once after the first): a wait in the
-            // first round alone makes the compiler peel it (34 -> 62 registers)
-            if (PDL && !DOT) grid_dep_wait();
+            // first round alone makes the compiler peel it (62 registers)
+            if (PDL && !DOT) grid_dep_sync();
             T xv[UNROLL];
 #pragma unroll
-            for (int u = 0; u < UNROLL; ++u) xv[u] = __ldg(x + cc[u]);
+            for (int u = 0; u < UNROLL; ++u) xv[u] = ldx(x + cc[u]);
 #pragma unroll
             for (int u = 0; u < UNROLL; ++u) t = fma(v[u], xv[u], t);
         }
-        for (; j < w; ++j) t = fma(__ldcs(vp + (int64_t)j * C), __ldg(x + __ldcs(cp + (int64_t)j * C)), t);
+        for (; j < w; ++j) t = fma(__ldcs(vp + (int64_t)j * C), ldx(x + __ldcs(cp + (int64_t)j * C)), t);
         const int io = orig_row(i, sigma, perm, perm_bytes);
         y[io] = t;
         if (DOT) {
-            d1 = fma(x[io], t, d1);
-            if (b) d2 = fma(x[io], b[io], d2);
+            const T xi = ldx(x + io);
+            d1 = fma(xi, t, d1);
+            if (b) d2 = fma(xi, ldx(b + io), d2);
         }
     }
     if (DOT) reduce_publish<sizeof(T) == 4>(red, (double)d1, (double)d2);
@@ -928,7 +932,10 @@ __global__ void __launch_bounds__(TPB)
                   const void *__restrict__ perm, int perm_bytes, const float *__restrict__ x,
                   float *__restrict__ y, Epilogue ep) {
     const int C = C32 ? 32 : Cr;  // a constant slot stride when C = 32
-    if (!EPI) grid_dep_launch();  // one pass over the rows: signal at block start
+    auto dep = [] {
+        grid_dep_wait();
+        if (!EPI) grid_dep_launch();
+    };
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) {
         grid_dep_wait();
@@ -951,18 +958,18 @@ __global__ void __launch_bounds__(TPB)
             cc[u] = ok ? __ldcs(cp + (int64_t)(j + u) * C) : -1;
         }
         if (!waited) {
-            grid_dep_wait();
+            dep();
             waited = true;
         }
         float xv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = cc[u] >= 0 ? __ldg(x + cc[u]) : 0.f;
+        for (int u = 0; u < U; ++u) xv[u] = cc[u] >= 0 ? ld_dep(x + cc[u]) : 0.f;
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (cc[u] >= 0) t = fmaf(__half2float(__ushort_as_half(v[u])), xv[u], t);
         if (cc[U - 1] < 0) break;  // padding: the row has ended
     }
-    if (!waited) grid_dep_wait();
+    if (!waited) dep();
     const int io = orig_row(i, sigma, perm, perm_bytes);
     y[io] = EPI ? epilogue(ep, x, io, t) : t;
 }

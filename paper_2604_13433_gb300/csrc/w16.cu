@@ -35,7 +35,6 @@ __global__ void __launch_bounds__(TPB, MINB)
                const void *__restrict__ perm, int perm_bytes, const float *__restrict__ x,
                float *__restrict__ y, int xlen) {
     const int C = C32 ? 32 : Cr;  // a constant word stride when C = 32
-    grid_dep_launch();  // one pass over the rows: signal at block start
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int k = i / C, l = i - k * C;
@@ -45,7 +44,7 @@ __global__ void __launch_bounds__(TPB, MINB)
     const int blk = sig_shift >= 0 ? (i >> sig_shift) << sig_shift : (i / sigma) * sigma;
     int c = (k_left < blk) ? (int)(blk - k_left) : 0;
     float t = 0.f;
-    if (w <= 0) grid_dep_wait();
+    if (w <= 0) grid_dep_sync();
     for (int j0 = 0; j0 < w; j0 += PF) {
         const int wr = w - j0;
         uint32_t wd[PF];
@@ -53,14 +52,14 @@ __global__ void __launch_bounds__(TPB, MINB)
         for (int u = 0; u < PF; ++u)
             wd[u] = (u < wr) ? (uint32_t)__ldcs(pp + (C32 ? (j0 + u) * 32 : (int64_t)(j0 + u) * C)) : 0u;
         // the first round's words load before the wait; x and y after it
-        if (j0 == 0) grid_dep_wait();
+        if (j0 == 0) grid_dep_sync();
         bool f[PF];
         float xv[PF];
 #pragma unroll
         for (int u = 0; u < PF; ++u) {
             f[u] = (wd[u] & 1u) != 0u;
             c += (int)((wd[u] >> 1) & (f[u] ? 0x7Fu : 0x7FFFu));
-            if (f[u]) xv[u] = PS_IN_RANGE(c, xlen) ? __ldg(x + c) : 0.f;
+            if (f[u]) xv[u] = PS_IN_RANGE(c, xlen) ? ld_dep(x + c) : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < PF; ++u)

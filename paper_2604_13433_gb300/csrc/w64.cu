@@ -31,7 +31,6 @@ __device__ __forceinline__ void w64_rows(int n, int C, int sigma, long long k_le
                                          const double *__restrict__ x, double *__restrict__ y,
                                          const double *__restrict__ b, Red red, int xlen) {
     if (DOT) grid_dep_sync();  // the reducing form waits before it starts
-    else grid_dep_launch();    // one pass over the rows: signal at block start
     if (DOT && red.sc->done) return;  // solver converged: idle (grid-uniform)
     // a decoded delta, and every column, stays below 2^31 (columns are int32 and
     // a dummy's delta is at most a column gap), so the delta comes from the low
@@ -47,13 +46,13 @@ __device__ __forceinline__ void w64_rows(int n, int C, int sigma, long long k_le
         const unsigned long long *pp = pack + s + l;
         int c = left_offset(i, sigma, k_left);
         double t = 0.0;
-        if (!DOT && w == 0) grid_dep_wait();
+        if (!DOT && w == 0) grid_dep_sync();
         for (int j0 = 0; j0 < w; j0 += WU) {
             unsigned long long wd[WU];
 #pragma unroll
             for (int u = 0; u < WU; ++u)
                 wd[u] = j0 + u < w ? __ldcs(pp + (int64_t)(j0 + u) * C) : 0ull;
-            if (!DOT) grid_dep_wait();  // returns at once after the first round
+            if (!DOT) grid_dep_sync();  // returns at once after the first round
             bool f[WU];
             double xv[WU];
 #pragma unroll
@@ -61,7 +60,7 @@ __device__ __forceinline__ void w64_rows(int n, int C, int sigma, long long k_le
                 const uint32_t lo = (uint32_t)wd[u];
                 f[u] = (lo & 1u) != 0u;
                 c += (int)((lo >> 1) & (f[u] ? dmask : 0x7fffffffu));
-                xv[u] = (f[u] && PS_IN_RANGE(c, xlen)) ? __ldg(x + c) : 0.0;
+                xv[u] = (f[u] && PS_IN_RANGE(c, xlen)) ? ld_dep(x + c) : 0.0;
             }
 #pragma unroll
             for (int u = 0; u < WU; ++u)
@@ -72,8 +71,9 @@ __device__ __forceinline__ void w64_rows(int n, int C, int sigma, long long k_le
         const int io = orig_row(i, sigma, perm, perm_bytes);
         y[io] = t;
         if (DOT) {
-            d1 = fma(x[io], t, d1);
-            if (b) d2 = fma(x[io], b[io], d2);
+            const double xi = ld_dep(x + io);
+            d1 = fma(xi, t, d1);
+            if (b) d2 = fma(xi, ld_dep(b + io), d2);
         }
     }
     if (DOT) reduce_publish<false>(red, d1, d2);
