@@ -53,10 +53,18 @@ inline int fgrid(int64_t n) {
 
 // sum of the block's FT values in shared memory by one warp (every lane has
 // it): 13 FP64 additions where a shuffle tree in all eight warps takes 40 (an
-// FP64 warp instruction takes about 16 cycles of an SM)
+// FP64 warp instruction takes about 16 cycles of an SM). With `err`, the
+// values' rounding errors are added too, a lane's in FP32 first (a second
+// rounding of 2^-24 of them): one more FP64 addition.
 template <typename T>
-__device__ __forceinline__ double warp_total(const T *v, int lane) {
+__device__ __forceinline__ double warp_total(const T *v, int lane, const float *err = nullptr) {
     double x[FT / 32], t = 0.0;
+    if (err) {
+        float e = 0.f;
+#pragma unroll
+        for (int q = 0; q < FT / 32; ++q) e += err[32 * q + lane];
+        t = (double)e;
+    }
 #pragma unroll
     for (int q = 0; q < FT / 32; ++q) x[q] = (double)v[32 * q + lane];
 #pragma unroll
@@ -271,17 +279,32 @@ __global__ void __launch_bounds__(FT) k_orth(int64_t n, const T *__restrict__ V,
 // registers through the dot products, the update and the scaling, and the
 // blocks (all resident: a cooperative launch) meet twice. Every block adds
 // all partials itself, in block order, so all have the same sums.
+// A thread's vectors are four elements wide, so it holds more products than a
+// thread of the separate kernels does, which add no two in FP32 up to 155,648
+// unknowns. Its products form four FP32 chains, one per place in the vector,
+// and the chains are added with their rounding error (two_sum): where a thread
+// has one vector (up to 622,592 unknowns) sum and error both enter the FP64
+// sums, and beyond that a chain is a quarter as long as a thread's chain in
+// the separate kernels. (One FP32 chain per thread: 64^3 unknowns 7.93 ms
+// instead of 8.03, 128^3 55.88 instead of 55.94.)
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {  // Knuth: a + b = sum + err
+    const float s = a + b, t = s - a;
+    err = (a - (s - t)) + (b - t);
+    return s;
+}
+
 template <int E>
 __global__ void __launch_bounds__(FT, 4)
     k_arnoldi(int64_t n, const float *__restrict__ V, int cnt, Hess h, int j, float *__restrict__ w,
               double *__restrict__ part, Meet m) {
     constexpr int PB = 8;  // quantities reduced together, one per warp
-    __shared__ float sh[PB][FT];
+    __shared__ float sh[PB][FT], sh_err[PB][FT];
     __shared__ float hf[64];
     __shared__ double s_norm;
     if (*(volatile int *)m.timeout) return;
     const int G = gridDim.x, wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t tid = blockIdx.x * (int64_t)FT + threadIdx.x, st = (int64_t)G * FT, nv = n / 4;
+    const bool one = nv <= st;  // at most one vector per thread
     float4 a[E / 4];
 #pragma unroll
     for (int k = 0; k < E / 4; ++k) {
@@ -309,11 +332,18 @@ __global__ void __launch_bounds__(FT, 4)
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         return s;
     };
+    // this thread's part of a quantity: its four chains and the tail's product
+    auto put = [&](int slot, float4 f, float ft) {
+        float e0, e1, e2, e3;
+        const float s = two_sum(two_sum(two_sum(f.x, f.y, e0), two_sum(f.z, f.w, e1), e2), ft, e3);
+        sh[slot][threadIdx.x] = s;
+        if (one) sh_err[slot][threadIdx.x] = (e0 + e1) + (e2 + e3);
+    };
     // the block's sums of the quantities [i0, i0 + count) in sh, one partial each
     auto block_parts = [&](int i0, int count, double *out) {
         __syncthreads();
         if (wl < count) {
-            const double s = warp_total(sh[wl], lane);
+            const double s = warp_total(sh[wl], lane, one ? sh_err[wl] : nullptr);
             if (lane == 0) out[(int64_t)(i0 + wl) * G + blockIdx.x] = s;
         }
         __syncthreads();
@@ -321,20 +351,20 @@ __global__ void __launch_bounds__(FT, 4)
     for (int i = 0; i < cnt; ++i) {
         const float *__restrict__ v = V + (int64_t)i * n;
         const bool al = ((uintptr_t)v & 15u) == 0;
-        float f = tail ? at * v[te] : 0.f;
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int k = 0; k < E / 4; ++k) {
             const int64_t q = tid + k * st;
             if (q < nv) {
                 const float4 b = al ? reinterpret_cast<const float4 *>(v)[q]
                                     : make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                f = fmaf(a[k].x, b.x, f);
-                f = fmaf(a[k].y, b.y, f);
-                f = fmaf(a[k].z, b.z, f);
-                f = fmaf(a[k].w, b.w, f);
+                f.x = fmaf(a[k].x, b.x, f.x);
+                f.y = fmaf(a[k].y, b.y, f.y);
+                f.z = fmaf(a[k].z, b.z, f.z);
+                f.w = fmaf(a[k].w, b.w, f.w);
             }
         }
-        sh[i % PB][threadIdx.x] = f;
+        put(i % PB, f, tail ? at * v[te] : 0.f);
         if (i % PB == PB - 1 || i + 1 == cnt) block_parts(i / PB * PB, i % PB + 1, part);
     }
     if (!meet(m, 1)) return;
@@ -364,15 +394,15 @@ __global__ void __launch_bounds__(FT, 4)
             }
         }
     }
-    float f = at * at;
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < E / 4; ++k) {
-        f = fmaf(a[k].x, a[k].x, f);
-        f = fmaf(a[k].y, a[k].y, f);
-        f = fmaf(a[k].z, a[k].z, f);
-        f = fmaf(a[k].w, a[k].w, f);
+        f.x = fmaf(a[k].x, a[k].x, f.x);
+        f.y = fmaf(a[k].y, a[k].y, f.y);
+        f.z = fmaf(a[k].z, a[k].z, f.z);
+        f.w = fmaf(a[k].w, a[k].w, f.w);
     }
-    sh[0][threadIdx.x] = f;
+    put(0, f, at * at);
     double *np = part + (int64_t)cnt * G;  // behind the dot products' partials
     block_parts(0, 1, np);
     if (!meet(m, 2)) return;
