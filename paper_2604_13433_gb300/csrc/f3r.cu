@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "device.cuh"
+#include "f3r_plan.h"
 #include "internal.h"
 #include "meet.cuh"
 
@@ -542,8 +543,7 @@ struct F3R {
     double *part;  // G * 64 partials
     unsigned *counter;  // blocks of the running reduction that have finished (0 between launches)
     Meet meet{};        // of k_arnoldi
-    int coop = 0;       // elements per thread of k_arnoldi (0: the three separate kernels)
-    int coop_blocks = 0;
+    StepPlan step;      // of the FP32 layers
     Layer<double> L1;
     Layer<TI> L2, L3;
     TI *rt = nullptr;  // the product of a Richardson step (the iterate is layer 3's z_j)
@@ -589,25 +589,32 @@ struct F3R {
         return PACKSELL_OK;
     }
 
-    // k_arnoldi's launch: all blocks resident, E elements of the vector per thread
-    template <int E>
-    bool plan_coop() {
-        int per = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arnoldi<E>, FT, 0) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        const int64_t most = (int64_t)device_sms() * std::min(per, 4);
-        const int64_t want = std::max<int64_t>(1, (n / 4 + FT - 1) / FT);  // one vector per thread
-        coop_blocks = (int)std::min(most, want);
-        if (coop_blocks < 1 || n / 4 > (int64_t)coop_blocks * FT * (E / 4)) return false;
-        coop = E;
-        return true;
+    // whether k_arnoldi runs, and on how many blocks; the trial launch finds
+    // the timeout flag set and returns at once
+    void plan_arnoldi() {
+        auto per_sm = [](int e) {
+            int per = 0;
+            const cudaError_t r = e == 16 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arnoldi<16>, FT, 0)
+                                          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arnoldi<32>, FT, 0);
+            if (r != cudaSuccess) cudaGetLastError();
+            return r == cudaSuccess ? per : 0;
+        };
+        auto fits = [&](int e, int blocks) {
+            step.blocks = blocks;
+            cudaError_t r = cudaMemsetAsync(meet.timeout, 0xff, sizeof(int), s);
+            if (r == cudaSuccess) {
+                Layer<float> none;
+                r = e == 16 ? launch_step<16>(none, nullptr, 0, 0) : launch_step<32>(none, nullptr, 0, 0);
+            }
+            if (r != cudaSuccess) cudaGetLastError();
+            return r == cudaSuccess;
+        };
+        step = plan_step(n, device_sms(), FT, per_sm, fits);
     }
 
     template <int E>
     cudaError_t launch_step(Layer<float> &L, float *w, int cnt, int j) {
-        return launch_coop(k_arnoldi<E>, (unsigned)coop_blocks, FT, 0, s, n, (const float *)L.V, cnt, L.h,
+        return launch_coop(k_arnoldi<E>, (unsigned)step.blocks, FT, 0, s, n, (const float *)L.V, cnt, L.h,
                            j, w, part, meet);
     }
 
@@ -620,8 +627,8 @@ struct F3R {
         if (st != PACKSELL_OK) return st;
         const int cnt = j + 1;
         if constexpr (std::is_same<T, float>::value) {
-            if (coop && ((uintptr_t)w & 15u) == 0) {
-                const cudaError_t e = coop == 16 ? launch_step<16>(L, w, cnt, j) : launch_step<32>(L, w, cnt, j);
+            if (step.elems && ((uintptr_t)w & 15u) == 0) {
+                const cudaError_t e = step.elems == 16 ? launch_step<16>(L, w, cnt, j) : launch_step<32>(L, w, cnt, j);
                 if (e != cudaSuccess) return cuda_fail(e, "f3r: Arnoldi step");
                 return PACKSELL_OK;
             }
@@ -721,7 +728,6 @@ packsell_status run_f3r(const Matrix &A1, const Matrix &A2, const Matrix &A3, co
     F.part = P.take<double>(64 * (size_t)G);
     F.counter = P.take<unsigned>(4);  // the reductions' counter; k_arnoldi's two and its flag
     F.meet = Meet{F.counter + 1, F.counter + 2, (int *)(F.counter + 3)};
-    if (std::is_same<TI, float>::value && !F.template plan_coop<16>()) F.template plan_coop<32>();
     r = P.take<double>(n);
     ax = P.take<double>(n);
     zt = P.take<double>(n);
@@ -733,6 +739,7 @@ packsell_status run_f3r(const Matrix &A1, const Matrix &A2, const Matrix &A3, co
         st = fail(PACKSELL_ERR_NO_MEMORY, "packsell_f3r: workspace carving");
         goto out;
     }
+    if (std::is_same<TI, float>::value) F.plan_arnoldi();
     {
         auto ck = [&](cudaError_t e) {
             if (e != cudaSuccess) st = cuda_fail(e, "packsell_f3r");
