@@ -258,6 +258,13 @@ packsell_status packsell_permute_csr(int64_t n, const int64_t *rowptr, const int
  * with no counterpart in the paper. */
 packsell_status packsell_destroy(packsell_matrix *A);
 
+/* The library keeps up to 2 GiB of freed device memory per device for its next
+ * calls, also after the last matrix is gone. This call synchronises the
+ * current device and returns what is unused to the system, for instance before
+ * another allocator needs it. Errors: CUDA (the device cannot be synchronised:
+ * a capture in progress). Housekeeping with no counterpart in the paper. */
+packsell_status packsell_trim(void);
+
 packsell_status packsell_get_info(const packsell_matrix *A, packsell_info *info);
 
 /* Serialise the stored arrays of §4.3 (no counterpart in the paper) to a

@@ -156,6 +156,12 @@ packsell_status packsell_destroy(packsell_matrix *A) {
     return PACKSELL_OK;
 }
 
+packsell_status packsell_trim(void) {
+    clear_error();
+    const cudaError_t e = pool_trim();
+    return e == cudaSuccess ? PACKSELL_OK : cuda_fail(e, "packsell_trim");
+}
+
 packsell_status packsell_get_info(const packsell_matrix *Ah, packsell_info *info) {
     clear_error();
     if (!Ah || !info) return fail(PACKSELL_ERR_INVALID_ARG, "packsell_get_info: NULL argument");

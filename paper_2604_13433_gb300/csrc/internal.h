@@ -114,6 +114,7 @@ cudaError_t pool_get(T **p, size_t bytes, cudaStream_t s) {
     return pool_get(reinterpret_cast<void **>(p), bytes, s);
 }
 void pool_put(void *p, cudaStream_t s);
+cudaError_t pool_trim();  // waits for the current device and returns what is unused to the system
 
 // How an object's arrays are given back: in the order of a stream. Every use of
 // them lies before on that stream, or the device has been synchronised.

@@ -7,7 +7,7 @@
 // middle) spent about 1 ms of its 1.4 ms in the allocator. The library's pool
 // keeps up to kKeep bytes of freed memory for the next call and returns the
 // rest to the system at the next synchronisation; when an allocation fails,
-// everything unused goes back and the allocation is tried once more.
+// and when the user asks for it (packsell_trim), everything unused goes back.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -64,13 +64,33 @@ cudaError_t pool_get(void **p, size_t bytes, cudaStream_t s) {
     bytes = bytes ? bytes : 16;
     e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     if (e == cudaErrorMemoryAllocation) {
+        // what is freed on any stream counts; a stream under capture must not be
+        // synchronised with
         cudaGetLastError();
-        flush_destroyed(dev);
-        cudaStreamSynchronize(s);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+            flush_destroyed(dev);
+            cudaDeviceSynchronize();
+        }
+        cudaGetLastError();
         cudaMemPoolTrimTo(pool, 0);
         e = cudaMallocFromPoolAsync(p, bytes, pool, s);
     }
     if (e == cudaSuccess) set_threshold(pool);
+    return e;
+}
+
+cudaError_t pool_trim() {
+    int dev = 0;
+    cudaMemPool_t pool;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) {
+        flush_destroyed(dev);
+        e = cudaDeviceSynchronize();
+    }
+    if (e == cudaSuccess) e = pool_of(dev, &pool);
+    if (e == cudaSuccess) e = cudaMemPoolTrimTo(pool, 0);
+    if (e != cudaSuccess) cudaGetLastError();
     return e;
 }
 

@@ -100,6 +100,7 @@ SIGNATURES = {
     "packsell_last_error": (ctypes.c_char_p, []),
     "packsell_encode": (ctypes.c_int, [_P, _I64, _I64, _I64, _P, _P, _P, _I32, _P, _P]),
     "packsell_destroy": (ctypes.c_int, [_P]),
+    "packsell_trim": (ctypes.c_int, []),
     "packsell_get_info": (ctypes.c_int, [_P, _P]),
     "packsell_export": (ctypes.c_int, [_P, _P, _P, _P]),
     "packsell_import": (ctypes.c_int, [_P, ctypes.c_size_t, _P, _P]),
@@ -228,6 +229,12 @@ class PackSELLMatrix:
 
 def packsell_version() -> str:
     return lib().packsell_version().decode()
+
+
+def packsell_trim() -> None:
+    """Return the device memory that the library keeps unused (up to 2 GiB per
+    device) to the system; synchronises the current device."""
+    _check(lib().packsell_trim())
 
 
 def packsell_encode(rowptr: torch.Tensor, col: torch.Tensor, val: torch.Tensor, n: int, m: int,
