@@ -403,12 +403,12 @@ def spmm_bytes(A, k):
     return 4 * A.n_words + 8 * (A.n_slices + 1) + perm + 4 * k * (A.m + A.n)
 
 
-def spmm_kernel(C, k):
-    """The kernel packsell_spmm runs for a C-row-slice matrix and k > 1 columns
-    (32-byte-aligned X and Y with k % 4 == 0, slices of at most 48 words when C = 32)."""
+def spmm_kernel(C, k, max_width=0):
+    """The kernel packsell_spmm runs for a matrix in slices of C rows and at most
+    max_width words per row, and k > 1 columns (32-byte-aligned X and Y with k % 4 == 0)."""
     if C == 1:
         return "k_split_rows" if k > 16 else "k_split_multi"
-    return "k_spmm_wide" if C == 32 and k % 8 == 0 else "k_spmm_packed"
+    return "k_spmm_wide" if C == 32 and k % 8 == 0 and max_width <= 48 else "k_spmm_packed"
 
 
 def irregular_section(ps, torch, dev, K, W, peak, n_rows=4194304):
@@ -454,7 +454,7 @@ def irregular_section(ps, torch, dev, K, W, peak, n_rows=4194304):
             Y = torch.empty(csr.n, k, device=dev)
             ms, _ = time_launches(torch, lambda: ps.packsell_spmm(M, X, Y), KS, 3)
             kern = (KERNEL_NAMES[ps.SPMV_SPLIT] if M.C == 1 else KERNEL_NAMES.get(v, "k_spmv")) \
-                if k == 1 else spmm_kernel(M.C, k)
+                if k == 1 else spmm_kernel(M.C, k, M.max_width)
             rows[str(k)] = _rate(spmm_bytes(M, k), ms, peak, kern,
                                  GFLOPs=2 * k * csr.nnz / ms / 1e6)
             del X, Y
@@ -500,7 +500,7 @@ def stencil_spmm_section(ps, torch, dev, K, peak):
         X = torch.rand(csr.m, k, device=dev)
         Y = torch.empty(csr.n, k, device=dev)
         ms, _ = time_launches(torch, lambda: ps.packsell_spmm(A, X, Y), KS, 3)
-        out[str(k)] = _rate(spmm_bytes(A, k), ms, peak, spmm_kernel(32, k),
+        out[str(k)] = _rate(spmm_bytes(A, k), ms, peak, spmm_kernel(A.C, k, A.max_width),
                             GFLOPs=2 * k * csr.nnz / ms / 1e6)
         del X, Y
     return out
