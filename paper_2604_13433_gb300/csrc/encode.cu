@@ -336,12 +336,13 @@ __global__ void __launch_bounds__(TPB)
                    int32_t *__restrict__ words, EncodeInfo *info) {
     __shared__ unsigned long long s_total;
     __shared__ int s_max;
-    if (info->st.code != 0) return;  // the counts are incomplete
     if (threadIdx.x == 0) {
         s_total = 0;
         s_max = 0;
     }
-    __syncthreads();
+    // the counts are incomplete. One answer for the block: another block may
+    // set the code between two warps' looks at it
+    if (__syncthreads_or(*(volatile int *)&info->st.code != 0)) return;
     unsigned long long v = 0;
     int longest = 0;
 #pragma unroll
