@@ -302,7 +302,8 @@ __global__ void __launch_bounds__(FT, 4)
     __shared__ float sh[PB][FT], sh_err[PB][FT];
     __shared__ float hf[64];
     __shared__ double s_norm;
-    if (*(volatile int *)m.timeout) return;
+    // (one answer for the block: another one may be setting the flag)
+    if (__syncthreads_or(*(volatile int *)m.timeout != 0)) return;
     const int G = gridDim.x, wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t tid = blockIdx.x * (int64_t)FT + threadIdx.x, st = (int64_t)G * FT, nv = n / 4;
     const bool one = nv <= st;  // at most one vector per thread
