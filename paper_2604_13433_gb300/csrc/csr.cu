@@ -215,8 +215,8 @@ void csr_plan_free(Matrix &A, const Release &rel) {
 
 // Items for variant 11 (C = 1 PackSELL matrices): consecutive rows of at
 // most CL words are grouped greedily while they hold at most CT words and CR
-// rows; a row of more than CL words is an item of its own. Built on the host
-// from the row offsets.
+// rows; a row of more than CL words is an item of its own. Cut on the device
+// from the row offsets (items.cu).
 CutRule csr_rule() { return CutRule{CUT_CSR, CL, CR}; }
 
 packsell_status launch_csr(const Matrix &A, const void *perm, int pb, const float *x, float *y,

@@ -431,16 +431,13 @@ __device__ __forceinline__ void rows_store(const SplitMat &M, float *__restrict_
     }
 }
 
-// words of a round per lane group. With two column groups per lane eight
+// Words of a round per lane group. With two column groups per lane eight
 // 16-byte gathers are in flight and the kernel runs two blocks per SM: 530 ->
 // 497 us at k = 64 on the power-law matrix of 1M rows, 127 -> 108 us on 60,000
 // rows (four gathers and three blocks before; a 4,096-word row is one warp's
 // work, 512 words' gathers one after another). With one group, four gathers
 // and three blocks (k = 32: 401 us; eight and two 403, eight and three 481).
-template <int NQ>
-constexpr int rows_round() {
-    return 4;
-}
+constexpr int kRowsRound = 4;
 
 // A tile: the words are split into RPI runs of about nwd / RPI words, each
 // moved forward to the next row start, so that every row lies in one run;
@@ -451,7 +448,7 @@ __device__ __forceinline__ void rows_tile(const SplitMat &M, int r0, int nrows, 
                                           int nwd, int lane, const uint4 &wv,
                                           uint32_t *__restrict__ s_lft, int *__restrict__ s_io,
                                           int4 *__restrict__ s_tab, const uint32_t *__restrict__ soff) {
-    constexpr int RPI = 32 / KG, U = rows_round<NQ>();
+    constexpr int RPI = 32 / KG, U = kRowsRound;
     const long long a0 = base & ~3ll;
     const int lead = (int)(base - a0);
     const uint32_t a0lo = (uint32_t)a0;
@@ -562,7 +559,7 @@ __device__ __forceinline__ void rows_tile(const SplitMat &M, int r0, int nrows, 
 template <int KG, int NQ>
 __device__ __forceinline__ void rows_long(const SplitMat &M, int row, long long base, int nwd,
                                           int lane, int4 *__restrict__ s_tab) {
-    constexpr int RPI = 32 / KG, U = rows_round<NQ>();
+    constexpr int RPI = 32 / KG, U = kRowsRound;
     static_assert(MT % (U * RPI) == 0, "a chunk splits evenly over the lane groups");
     const long long a0 = base & ~3ll;
     const int lead = (int)(base - a0), lim = lead + nwd;

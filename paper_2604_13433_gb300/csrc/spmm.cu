@@ -328,7 +328,12 @@ packsell_status spmm_impl(const Matrix &A, int k, const float *X, int64_t ldx, f
                                                 vec, s);
         return st;
     }
-    // 32-byte rows and slices of at most 48 words: eight columns per lane
+    // 32-byte rows and slices of at most 48 words: eight columns per lane. The
+    // limit is not where the form stops paying: on rows of 24 to 256 words, even
+    // and uneven, near the diagonal and 64 columns apart, it takes less time than
+    // the kernel below at each of k = 8, 16 and 64 (48 words, 500,000 even rows,
+    // k = 64: 257 against 366 us; 64 words 256 / 349, 256 words 271 / 330). Longer
+    // rows, such as a power-law matrix's of up to 4,096 words, are not measured.
     if (A.p.C == 32 && is_packed(A.p.format) && A.max_width <= 48 && k % 8 == 0 && ldx % 8 == 0 &&
         ldy % 8 == 0 && ldx < (1ll << 30) && ((uintptr_t)X & 31) == 0 && ((uintptr_t)Y & 31) == 0) {
         if (A.p.format == PACKSELL_FMT_FP16)
