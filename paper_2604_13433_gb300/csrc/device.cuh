@@ -135,18 +135,6 @@ __device__ __forceinline__ __half ld_dep(const __half *p) {
     asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
     return __ushort_as_half(v);
 }
-__device__ __forceinline__ float4 ld_dep(const float4 *p) {
-    float4 v;
-    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "l"(p));
-    return v;
-}
-__device__ __forceinline__ double2 ld_dep(const double2 *p) {
-    double2 v;
-    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
-    return v;
-}
 
 // One word: add its delta to c; if it carries a value, gather x_c (DEP: in a
 // kernel started by launch_pdl).
